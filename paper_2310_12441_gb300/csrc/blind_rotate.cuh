@@ -136,14 +136,15 @@ __device__ __forceinline__ void mmpm_row(u32 c, u32 i, u32 m, u32 twoN, u32 gS, 
 //    lands on coefficient j = (a S + E_s) mod N, negated when
 //    (a S + E_s) mod 2N >= N; so coefficient j holds the term
 //    a = (j - E_s) S^-1 mod N.
-// Rows i with i mod rows_step == row0 only (the rows of one block of a cluster).
+// Rows i with i mod rows_step == row0 only (the rows of one block of a cluster),
+// by `threads` threads of which this is number tid.
 static __device__ void acc_init(u64 *__restrict__ acc, const u32 *__restrict__ lut, u64 b, u32 m, u32 t,
                                 u32 N, u64 Q, u32 gS, u32 gSinv, const u32 *pre, u32 row0 = 0,
-                                u32 rows_step = 1) {
+                                u32 rows_step = 1, u32 tid = threadIdx.x, u32 threads = blockDim.x) {
     const u64 qp = 2ull * N * m;
     const u64 dq = Q / t;
     const u32 twoN = 2 * N;
-    for (u32 idx = threadIdx.x; idx < m * 2 * N; idx += blockDim.x) {
+    for (u32 idx = tid; idx < m * 2 * N; idx += threads) {
         const u32 c = idx % N;
         const u32 comp = (idx / N) & 1;
         const u32 i = idx / (2 * N);
@@ -282,8 +283,9 @@ __device__ __forceinline__ void br_job(const DevJob &J, u32 steps_limit, const u
     constexpr int R = C::R;
     constexpr int N = C::N, G = C::G, CPB = C::CPB;
     const KeyDev *K = J.key;
-    // (keys of the Q = c 2^32 + 1 kernels have 30-bit limbs: choose_variant)
-    const u32 lbits = QLOW1 ? 30u : J.lbits;
+    // (keys of the Q = c 2^32 + 1 kernels have limbs of a fixed width)
+    constexpr u32 LB = br_qlow1_limb(LAZY);
+    const u32 lbits = QLOW1 ? LB : J.lbits;
     const bool fold_each = J.fold_each != 0;
     const u32 m = J.m, t = J.t, lB = K->l_B, log2B = K->log2_B, n = K->n;
     const ModQ mq = K->mq;
@@ -348,8 +350,11 @@ __device__ __forceinline__ void br_job(const DevJob &J, u32 steps_limit, const u
     const size_t rgsw = (size_t)2 * lB * 2 * N;
 
     // Limb products of a transform value xv with the key words of the two
-    // columns: x1 b1, x0 b0 and (x0 + x1)(b0 + b1) accumulate with
-    // mad.wide.u32 (one multiplier instruction each, the addition included).
+    // columns: x1 b1, x0 b0 and (x0 + x1)(b0 + b1).  A wide product with a
+    // 64-bit addend holds the multiplier about 5 cycles per warp, one without
+    // 2 and its addition goes to the integer ALU: four of the six as product
+    // and addition balance the two pipes (22.8 cycles per value and SM
+    // sub-partition against 39.7 with six mad.wide, 25.8 with none).
     // xv's limbs are split once (funnel shift: lbits <= 31 and xv <
     // 2^(lbits + 32)) for both columns.  The key stores per position the low
     // limbs of both columns in w0 and their high limbs in w1 (32-bit halves),
@@ -358,23 +363,23 @@ __device__ __forceinline__ void br_job(const DevJob &J, u32 steps_limit, const u
     const u32 lmask32 = (u32)lmask;
     auto kara2 = [&](u64 xv, u64 w0, u64 w1, u64 (&kh)[2], u64 (&kl)[2], u64 (&km)[2]) {
         if constexpr (QLOW1) {
-            asm("{\n\t.reg .u32 v0, v1, x0, x1, xs, a0, a1, as, c0, c1, cs;\n\t.reg .u64 s;\n\t"
+            asm("{\n\t.reg .u32 v0, v1, x0, x1, xs, a0, a1, as, c0, c1, cs;\n\t.reg .u64 s, t;\n\t"
                 "mov.b64 {v0, v1}, %6;\n\t"
-                "shf.r.clamp.b32 x1, v0, v1, 30;\n\t"
-                "and.b32 x0, v0, 1073741823;\n\t"
+                "shf.r.clamp.b32 x1, v0, v1, %9;\n\t"
+                "and.b32 x0, v0, %10;\n\t"
                 "add.u32 xs, x0, x1;\n\t"
                 "mov.b64 {a0, c0}, %7;\n\t"
                 "mov.b64 {a1, c1}, %8;\n\t"
                 "add.u64 s, %7, %8;\n\t"
                 "mov.b64 {as, cs}, s;\n\t"
-                "mad.wide.u32 %0, x1, a1, %0;\n\t"
+                "mul.wide.u32 t, x1, a1;\n\tadd.u64 %0, %0, t;\n\t"
                 "mad.wide.u32 %1, x0, a0, %1;\n\t"
-                "mad.wide.u32 %2, xs, as, %2;\n\t"
-                "mad.wide.u32 %3, x1, c1, %3;\n\t"
+                "mul.wide.u32 t, xs, as;\n\tadd.u64 %2, %2, t;\n\t"
+                "mul.wide.u32 t, x1, c1;\n\tadd.u64 %3, %3, t;\n\t"
                 "mad.wide.u32 %4, x0, c0, %4;\n\t"
-                "mad.wide.u32 %5, xs, cs, %5;\n\t}"
+                "mul.wide.u32 t, xs, cs;\n\tadd.u64 %5, %5, t;\n\t}"
                 : "+l"(kh[0]), "+l"(kl[0]), "+l"(km[0]), "+l"(kh[1]), "+l"(kl[1]), "+l"(km[1])
-                : "l"(xv), "l"(w0), "l"(w1));
+                : "l"(xv), "l"(w0), "l"(w1), "n"(LB), "n"((1u << LB) - 1));
             return;
         }
         asm("{\n\t.reg .u32 v0, v1, x0, x1, xs, a0, a1, as, c0, c1, cs;\n\t.reg .u64 s;\n\t"

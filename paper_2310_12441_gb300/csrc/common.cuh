@@ -53,6 +53,11 @@ struct DevJob {
 #define BR_V_QLOW1 1u   // Q = c 2^32 + 1: one-multiply q Q
 #define BR_V_LAZY 2u    // correction-free forward NTT with an exact first stage
 
+// Limb width of the keys with Q = c 2^32 + 1: 28 bits for the lazy ones (their
+// transform values are below 2^60, their key words below 2^55: a short high
+// key limb lets more products fit 64 bits), 30 for the others.
+__host__ __device__ constexpr u32 br_qlow1_limb(bool lazy) { return lazy ? 28u : 30u; }
+
 // Arithmetic variant of a key set (BR_V_* flags):
 //  - BR_V_QLOW1: Q = c 2^32 + 1 < 2^60;
 //  - BR_V_LAZY: the correction-free forward transform.  With Q = c 2^32 + 1
@@ -68,9 +73,10 @@ inline u32 choose_variant(const bm_key_params &p) {
     u32 v = 0;
     // (Q < 2^60 keeps every value the Q = c 2^32 + 1 butterflies correct below 2^63)
     bool qlow1 = (p.Q & 0xffffffffull) == 1 && p.Q < (1ull << 60);
-    // the Q = c 2^32 + 1 kernels also fix the multiply-accumulate's limbs at
-    // 30 bits (limb_plan: the transform outputs' bound below 2^60, above 2^58)
-    const bool lazy1 = (1 + 4 * (u128)logN) * Q < ((u128)1 << 62) && 128 * Q < lim;
+    // the Q = c 2^32 + 1 kernels also fix the multiply-accumulate's limbs
+    // (br_qlow1_limb): the transform outputs' bound above 2^58 and below 2^60,
+    // for the lazy ones low enough that their limb sums fit 32 bits
+    const bool lazy1 = (1 + 4 * (u128)logN) * Q < ((u128)15 << 56) && 128 * Q < lim;
     const u128 xmax1 = lazy1 ? (1 + 4 * (u128)logN) * Q : Q;
     if (qlow1 && !(xmax1 - 1 >= ((u128)1 << 58) && xmax1 - 1 < ((u128)1 << 60))) qlow1 = false;
     if (qlow1) {
@@ -88,7 +94,8 @@ inline u32 choose_variant(const bm_key_params &p) {
 // products x1 b1, x0 b0, (x0 + x1)(b0 + b1) of a batch of CPB combos are
 // summed in 64-bit registers.  xmax is where the forward transform leaves
 // its outputs (ntr::fwd_to_smem): (1 + 4 log2 N) Q (lazy, Q = c 2^32 + 1,
-// unreduced), 2Q (lazy), Q.  lbits = ceil(bits(xmax - 1) / 2); fold_each when
+// unreduced), 2Q (lazy), Q.  lbits = ceil(bits(xmax - 1) / 2), or the fixed
+// width of the Q = c 2^32 + 1 kernels; fold_each when
 // CPB times the largest middle product could reach 2^64 (then each combo is
 // folded at once).  The key stores every BSK word b pre-split as
 // (b mod 2^lbits) | (b >> lbits) 2^32.
@@ -100,7 +107,7 @@ inline void limb_plan(const bm_key_params &p, u32 variant, u32 &lbits, u32 &fold
                                             : (u128)p.Q;
     u32 bits = 0;
     while (bits < 66 && ((xmax - 1) >> bits)) bits++;
-    lbits = (bits + 1) / 2;
+    lbits = (variant & BR_V_QLOW1) ? br_qlow1_limb((variant & BR_V_LAZY) != 0) : (bits + 1) / 2;
     const u128 lim = (u128)1 << lbits;
     const u128 sx = (lim - 1) + ((xmax - 1) >> lbits), sb = (lim - 1) + ((u128)(p.Q - 1) >> lbits);
     const u32 cpb = 512u / (p.N / 16u);     // the largest CPB of any kernel shape
