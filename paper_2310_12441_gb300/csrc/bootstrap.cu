@@ -476,6 +476,9 @@ u32 log2u(u32 N) {
 bm_status launch_br_any(u32 N, u32 variant, u32 shape, const DevJob *jobs, uint32_t cnt, u32 mmax, u32 max_cluster,
                     u32 steps, const uint64_t *ct_in, const uint32_t *lut, u64 *ws_acc, u32 *status,
                     cudaStream_t st, bool dry) {
+    if (shape == 1 && (variant & (BR_V_TC1 | BR_V_TC2)))
+        return bm_launch_br_tc(N, variant, jobs, cnt, mmax, max_cluster, steps, ct_in, lut, ws_acc, status,
+                               status + BM_WS_GROUP_WORD, 0, st, dry);
     switch (N) {
         case 256:
         case 512:

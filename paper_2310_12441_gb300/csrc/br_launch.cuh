@@ -169,7 +169,7 @@ bm_status launch_br(u32 variant, u32 shape, const DevJob *jobs, uint32_t cnt, u3
                     bool dry) {
 #define BM_LAUNCH(LZ, S0, QL) \
     return launch_shape<LOGN, LZ, S0, QL>(shape, jobs, cnt, mmax, max_cluster, steps, ct_in, lut, ws_acc, status, st, dry)
-    switch (variant) {
+    switch (variant & BR_V_ARITH) {
         case BR_V_LAZY | BR_V_QLOW1: BM_LAUNCH(true, true, true);
         case BR_V_LAZY: BM_LAUNCH(true, true, false);
         case BR_V_QLOW1: BM_LAUNCH(false, true, true);

@@ -24,6 +24,10 @@ struct KeyDev {
     const u64 *itwsh;
     const u64 *twp;    // forward (twiddle, companion) pairs, 16-byte aligned
     const u64 *itwp;   // inverse pairs
+    const void *tc;    // tables of the tensor-core transform stages (tc_tables), or null
+    u32 tc_t0, tc_m;   // their quotient constants
+    u64 tc_b1, tc_b1s, tc_b2, tc_b2s;   // 2^LB, 2^(2 LB) mod Q (LB the limb width) and companions
+    u32 tc_fs, tc_fsh; // floor(v / Q) for v < 2^64, at most one below: (v >> 32) tc_fs >> (32 + tc_fsh)
     ModQ mq;
     u64 ninv, ninv_sh; // N^-1 mod Q and companion
     u64 ks_pq;         // floor(P 2^64 / Q), P = B_ks^l_ks
@@ -52,6 +56,9 @@ struct DevJob {
 // Arithmetic variants of the blind rotation, chosen per key set on the host.
 #define BR_V_QLOW1 1u   // Q = c 2^32 + 1: one-multiply q Q
 #define BR_V_LAZY 2u    // correction-free forward NTT with an exact first stage
+#define BR_V_TC1 4u     // leading transform stages on the tensor cores (br_tc.cuh), limb
+#define BR_V_TC2 8u     // configuration 1 or 2
+#define BR_V_ARITH 3u   // the flags of the CUDA-core kernels
 
 // Limb width of the keys with Q = c 2^32 + 1: 28 bits for the lazy ones (their
 // transform values are below 2^60, their key words below 2^55: a short high
@@ -86,6 +93,15 @@ inline u32 choose_variant(const bm_key_params &p) {
                128 * Q < lim) {
         v |= BR_V_LAZY;
     }
+    // The tensor-core stages (br_tc.cuh): digits of at most 10 bits (9 at N =
+    // 1024), the digits of two (sign, component) pairs (N = 1024) or one (N =
+    // 2048) in whole half batches, within the shared memory beside the weights.
+    // Every such key gains (one bootstrap at N = 1024: 18.6 ms without, 15.4 with
+    // them; full blocks as in br_tc.cuh), so no size is left to the other form.
+    const bool tc1 = p.Q < (1ull << 54) && p.log2_B <= 9;
+    if ((v & BR_V_QLOW1) && p.l_B <= 6 && p.l_B % 2 == 0 && p.log2_B <= 10 &&
+        ((p.N == 1024 && (v & BR_V_LAZY) && tc1) || p.N == 2048))
+        v |= tc1 ? BR_V_TC1 : BR_V_TC2;
     return v;
 }
 
@@ -116,9 +132,11 @@ inline void limb_plan(const bm_key_params &p, u32 variant, u32 &lbits, u32 &fold
     fold_each = (u128)cpb * sx * sb >= ((u128)1 << 64);
 }
 
-// Workspace header: [0] status word, [1 + c] job counter of persistent class c.
+// Workspace header: [0] status word, [1 + c] job counter of persistent class c,
+// [BM_WS_GROUP_WORD] job counter of a grouped launch.
 #define BM_WS_COUNTER_WORD 1
 #define BM_MAX_CLASSES 15
+#define BM_WS_GROUP_WORD 16
 
 // Host-side evaluation key.
 struct bm_eval_key {
@@ -128,6 +146,7 @@ struct bm_eval_key {
     KeyDev host_view;  // same fields as the device copy (pointers are device pointers)
     KeyDev *d_view;
     u64 *d_bsk, *d_ksk, *d_tables;
+    void *d_tc;        // tensor-core tables (null without them)
     size_t bytes;
 };
 
@@ -189,6 +208,13 @@ bm_status bm_big_poly_mul(const u64 *a, const u64 *b, uint32_t count, u64 *out, 
                           u64 Q, u32 N, cudaStream_t st);
 bm_status bm_launch_br_big(u32 N, const DevJob *jobs, uint32_t cnt, u32 steps, const uint64_t *ct_in,
                            const uint32_t *lut, u64 *ws_acc, u32 *status, cudaStream_t st);
+
+// Tensor-core form (br_tc.cu), ring degrees 1024 and 2048 of keys with a
+// BR_V_TC* flag: grouped launches and persistent classes (max_cluster = 1);
+// counter: the jobs' counter, a word of the workspace header; sms 0: look up.
+bm_status bm_launch_br_tc(u32 N, u32 variant, const DevJob *jobs, uint32_t cnt, u32 mmax, u32 max_cluster, u32 steps,
+                          const uint64_t *ct_in, const uint32_t *lut, u64 *ws_acc, u32 *status, u32 *counter, int sms,
+                          cudaStream_t st, bool dry);
 
 // Host helpers (keygen.cu)
 bm_status bm_check_key_params(const bm_key_params *p);

@@ -81,7 +81,7 @@ template <int LOGN>
 bm_status launch_variant(u32 variant, u32 shape, const DevJob *d_jobs, uint32_t count, uint32_t steps,
                          const uint64_t *ct_in, const uint32_t *lut, u64 *ws_acc, u32 *status, u32 *counter, int sms,
                          bool dry, cudaStream_t st) {
-    switch (variant) {
+    switch (variant & BR_V_ARITH) {
         case BR_V_LAZY | BR_V_QLOW1:
             return launch_class_shape<LOGN, BR_V_LAZY | BR_V_QLOW1>(shape, d_jobs, count, steps, ct_in, lut, ws_acc,
                                                                    status, counter, sms, dry, st);
@@ -106,6 +106,9 @@ bm_status bm_launch_persistent_class(u32 N, u32 variant, u32 shape, const DevJob
                                      u32 *status, u32 *counter, int device, bool dry, cudaStream_t st) {
     int sms = 0;
     BM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
+    if (shape == 1 && (variant & (BR_V_TC1 | BR_V_TC2)))
+        return bm_launch_br_tc(N, variant, d_jobs, count, 1, 1, steps, ct_in, lut, ws_acc, status, counter, sms, st,
+                               dry);
     switch (N) {
         case 1024:
             return launch_variant<10>(variant, shape, d_jobs, count, steps, ct_in, lut, ws_acc, status, counter, sms,
