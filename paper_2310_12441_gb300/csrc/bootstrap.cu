@@ -25,22 +25,11 @@
 #include "ntt_reg.cuh"
 
 #include "br_launch.cuh"
+#include "ks_tile.cuh"
 
 // ---------------------------------------------------------------------------
 // Sample extraction + key switching
 // ---------------------------------------------------------------------------
-
-// a~ = floor((a P + floor(Q/2)) / Q) mod P, exact: the Shoup-style quotient
-// estimate floor(a P' / 2^64), P' = floor(P 2^64 / Q), is at most 2 below the
-// true quotient; the remainder fits in 64 bits and fixes it.
-__device__ __forceinline__ u64 ks_round(u64 a, const KeyDev &K) {
-    const u32 sh = K.log2_Bks * K.l_ks;
-    const u64 Q = K.mq.Q;
-    u64 q = __umul64hi(a, K.ks_pq);
-    u64 r = (a << sh) + Q / 2 - q * Q;
-    for (int it = 0; it < 3 && r >= Q; it++) { r -= Q; q++; }
-    return q & ((1ull << sh) - 1);
-}
 
 // Address of `p` (this block's shared memory) in the shared memory of block
 // `rank` of the cluster (distributed shared memory), and a load from it.
@@ -76,11 +65,19 @@ __device__ void key_switch_block(const KeyDev &K, GetA get_a, u64 b, u64 *__rest
     u64 lo[CPT], hi[CPT];
 #pragma unroll
     for (int q = 0; q < CPT; q++) lo[q] = hi[q] = 0;
-    const size_t rowlen = n + 1;
+    const size_t coef = (size_t)lks * B1 * ksk_pitch(n);     // words of a coefficient
+    u32 col[CPT], width[CPT];      // this thread's columns within a coefficient, the width of their slices
+#pragma unroll
+    for (int q = 0; q < CPT; q++) {
+        const u32 c = threadIdx.x + q * blockDim.x, c0 = c & ~(kKskCols - 1);
+        width[q] = c <= n ? ksk_slice_width(n, c0) : 0;
+        col[q] = c0 * lks * B1 + c - c0;
+    }
     const u32 rows = (i1 - i0) * lks;
     constexpr int KR = CPT == 4 ? 4 : 2;
     for (u32 r0 = 0; r0 < rows; r0 += KR) {
-        const u64 *rp[KR];
+        const u64 *cp[KR];
+        u32 row[KR];
         bool ok[KR];
 #pragma unroll
         for (int k = 0; k < KR; k++) {
@@ -88,7 +85,8 @@ __device__ void key_switch_block(const KeyDev &K, GetA get_a, u64 b, u64 *__rest
             const u32 d = rr < rows ? dsm[rr] : 0;    // digit d_ij of row rr = (i - i0) lks + j
             ok[k] = d != 0;
             const u32 i = i0 + rr / lks, j = rr % lks;
-            rp[k] = K.ksk + (((size_t)i * lks + j) * B1 + (ok[k] ? d - 1 : 0)) * rowlen;
+            cp[k] = K.ksk + i * coef;
+            row[k] = j * B1 + d - 1;
         }
         u64 v[KR][CPT];
 #pragma unroll
@@ -96,7 +94,7 @@ __device__ void key_switch_block(const KeyDev &K, GetA get_a, u64 b, u64 *__rest
 #pragma unroll
             for (int q = 0; q < CPT; q++) {
                 const u32 c = threadIdx.x + q * blockDim.x;
-                v[k][q] = (ok[k] && c <= n) ? __ldg(rp[k] + c) : 0;
+                v[k][q] = (ok[k] && c <= n) ? __ldg(cp[k] + (col[q] + row[k] * width[q])) : 0;
             }
 #pragma unroll
         for (int k = 0; k < KR; k++)
@@ -153,6 +151,51 @@ __global__ void BM_KS_BOUNDS(CPT) k_key_switch(const KeyDev *Kp, const u64 *__re
     const u64 *in = lwe_in + job * (K.N + 1);
     auto get_a = [&](u32 i) -> u64 { return in[i]; };
     key_switch_block<CPT>(K, get_a, in[K.N], out + job * (K.n + 1), rank, S);
+}
+
+// Tiles of samples (ks_tile.cuh): block = tile blockIdx.x / slices, column
+// slice blockIdx.x mod slices; jobs / samples 0 .. count - 1 have one key.
+template <int CPT>
+__global__ void __launch_bounds__(kst::kThreads, 1)
+    k_extract_keyswitch_tile(const DevJob *__restrict__ jobs, u32 count, u32 slices, u32 steps_limit,
+                             const u64 *__restrict__ ws, u64 *__restrict__ ct_out, u32 *status) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    const KeyDev &K = *jobs[0].key;
+    const u32 N = K.N;
+    const u64 Q = K.mq.Q;
+    const u32 steps = steps_limit < K.n ? steps_limit : K.n;
+    auto acc_of = [&](u32 s) { return ws + jobs[s].acc_off + ((steps & 1) ? (size_t)jobs[s].m * 2 * N : 0); };
+    auto load = [&](u32 s, u32 i, u64 (&v)[kst::kGroup]) {
+        const u64 *acc = acc_of(s);
+#pragma unroll
+        for (u32 g = 0; g < kst::kGroup; g++) {
+            const u64 a = acc[i + g ? N - i - g : 0];
+            v[g] = i + g && a ? Q - a : a;
+        }
+    };
+    auto store = [&](u32 s, u32 c, u64 sum, bool failed) {
+        ct_out[jobs[s].out_off + c] = failed ? ~0ull : sub_mod(c == K.n ? acc_of(s)[N] : 0, sum, Q);
+    };
+    kst::tile<CPT>(K, blockIdx.x / slices * CPT * kst::kWarpsPer, count, blockIdx.x % slices * kKskCols, dsm, load,
+                   store, status);
+}
+
+template <int CPT>
+__global__ void __launch_bounds__(kst::kThreads, 1)
+    k_key_switch_tile(const KeyDev *Kp, u32 count, u32 slices, const u64 *__restrict__ lwe_in, u64 *__restrict__ out) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    const KeyDev &K = *Kp;
+    auto load = [&](u32 s, u32 i, u64 (&v)[kst::kGroup]) {
+        const u64 *in = lwe_in + (size_t)s * (K.N + 1) + i;
+#pragma unroll
+        for (u32 g = 0; g < kst::kGroup; g++) v[g] = in[g];
+    };
+    auto store = [&](u32 s, u32 c, u64 sum, bool failed) {
+        const u64 b = c == K.n ? lwe_in[(size_t)s * (K.N + 1) + K.N] : 0;
+        out[(size_t)s * (K.n + 1) + c] = failed ? ~0ull : sub_mod(b, sum, K.mq.Q);
+    };
+    kst::tile<CPT>(K, blockIdx.x / slices * CPT * kst::kWarpsPer, count, blockIdx.x % slices * kKskCols, dsm, load,
+                   store, nullptr);
 }
 
 __global__ void k_sample_extract(const KeyDev *Kp, const u64 *__restrict__ rlwe, u64 *__restrict__ lwe) {
@@ -549,10 +592,17 @@ struct Fork {
     std::vector<cudaEvent_t> ev;      // [0] fork, [1 + c] join of side stream c
 };
 
+// What the key switch's launch rule needs of a key.
+struct KsKey {
+    const KeyDev *dev;
+    u32 N, n, lks, log2_Bks;
+};
+
 struct KsShape {
     u32 threads, cpt;
     size_t smem;   // digits of all N coefficients (one block per job) + partial sums
     u32 maxN, maxlks, maxn;
+    std::vector<KsKey> keys;
     // shared memory when S blocks split a job's coefficients
     size_t smem_for(u32 S) const { return align_up((size_t)(maxN / S) * maxlks, 16) + 8 * (size_t)(maxn + 1); }
 };
@@ -565,6 +615,8 @@ KsShape ks_shape(const bm_eval_key *const *keys, uint32_t n_keys) {
         maxlks = keys[i]->p.l_ks > maxlks ? keys[i]->p.l_ks : maxlks;
     }
     KsShape k;
+    for (uint32_t i = 0; i < n_keys; i++)
+        k.keys.push_back({keys[i]->d_view, keys[i]->p.N, keys[i]->p.n, keys[i]->p.l_ks, keys[i]->p.log2_Bks});
     k.cpt = maxn + 1 <= 1024 ? 4 : 8;
     k.threads = k.cpt == 4 ? 256 : ((maxn + 1 + 7) / 8 + 31) / 32 * 32;
     k.maxN = maxN;
@@ -584,8 +636,8 @@ u32 ks_split(uint32_t count, int device) {
     return S;
 }
 
-template <typename Kern, typename... Args>
-bm_status launch_ks_kernel(Kern kern, uint32_t count, u32 S, const KsShape &ks, cudaStream_t st, Args... args) {
+template <auto kern, typename... Args>
+bm_status launch_ks_kernel(uint32_t count, u32 S, const KsShape &ks, cudaStream_t st, Args... args) {
     static std::atomic<uint64_t> attr_done{0};
     bm_status s = ensure_smem(kern, 96 * 1024, attr_done);
     if (s != BM_OK) return s;
@@ -615,11 +667,94 @@ bm_status launch_ks_kernel(Kern kern, uint32_t count, u32 S, const KsShape &ks, 
     return BM_OK;
 }
 
-bm_status launch_extract_ks(const KsShape &ks, uint32_t count, u32 S, cudaStream_t st, const DevJob *d_jobs,
-                            u32 steps, const u64 *ws_acc, uint64_t *d_out) {
-    if (ks.cpt == 4)
-        return launch_ks_kernel(k_extract_keyswitch<4>, count, S, ks, st, d_jobs, steps, ws_acc, d_out);
-    return launch_ks_kernel(k_extract_keyswitch<8>, count, S, ks, st, d_jobs, steps, ws_acc, d_out);
+// Samples per thread of the tiled key switch for `count` samples of one key,
+// 0: one block (cluster) per sample.  The cheaper of the two by times measured
+// for l_ks = 3..16, B_ks = 2..128, n = 64..1030, 80..2049 samples, in cycles per
+// coefficient of the ring.  A tile: 700 per stage, 50 and 36 per sample of a
+// thread for every digit, at least its key rows at 64 B per cycle.  A block per
+// sample: per digit 230 (n < 256) or 340, 370 with more blocks than SMs (latency),
+// or for every sample 1/8 per column slice, at least 9/8 (throughput).  Up to
+// half the SMs a cluster per sample is faster (n = 630, N = 1024: 64 samples
+// 0.68 ms against 1.08; 96: 1.32 against 1.08; 2000: 9.6 against 3.2; B_ks = 128,
+// n = 830, N = 256: 300 samples 0.24 against 0.52, 2049: 1.44 against 0.81).
+u32 ks_tile_cpt(const KsKey &k, uint32_t count, u32 sms) {
+    const u32 jn = kst::digits_per_stage(k.lks, k.log2_Bks);
+    if (jn == 0 || 2ull * count <= sms) return 0;
+    const u32 slices = (k.n + kKskCols) / kKskCols, parts = (k.lks + jn - 1) / jn;
+    const u64 fill = (u64)k.lks * ((1u << k.log2_Bks) - 1) * kKskCols * 8 / 64;
+    const u64 latency = count > sms ? 370 : k.n < 256 ? 230 : 340;
+    u64 best_cost = k.lks * std::max<u64>(latency, (u64)count * std::max(slices, 9u) / 8);
+    u32 best = 0;
+    for (u32 cpt = 4; cpt <= kst::kMaxCpt; cpt += 4) {
+        if (kst::smem_bytes(k.lks, k.log2_Bks, cpt * kst::kWarpsPer, 2) > kst::kMaxSmem) break;
+        const u64 tiles = (count + cpt * kst::kWarpsPer - 1) / (cpt * kst::kWarpsPer);
+        const u64 waves = (tiles * slices + sms - 1) / sms;
+        const u64 cost = waves * std::max<u64>(700 * parts + k.lks * (50 + 36 * cpt), fill);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = cpt;
+        }
+    }
+    return best;
+}
+
+template <auto kern, typename... Args>
+bm_status launch_ks_tile(u32 cpt, const KsKey &k, uint32_t count, cudaStream_t st, Args... args) {
+    static std::atomic<uint64_t> attr_done{0};
+    bm_status s = ensure_smem(kern, kst::kMaxSmem, attr_done);
+    if (s != BM_OK) return s;
+    const u32 slices = (k.n + kKskCols) / kKskCols, per = cpt * kst::kWarpsPer;
+    kern<<<(count + per - 1) / per * slices, kst::kThreads,
+           kst::smem_bytes(k.lks, k.log2_Bks, per, kst::stages_of(k.lks, k.log2_Bks, per)), st>>>(args...);
+    BM_CUDA_TRY(cudaGetLastError());
+    return BM_OK;
+}
+
+#define BM_KS_TILE(KERN, CPT, ...)                                             \
+    switch (CPT) {                                                             \
+        case 4: return launch_ks_tile<KERN<4>>(4, __VA_ARGS__);                \
+        case 8: return launch_ks_tile<KERN<8>>(8, __VA_ARGS__);                \
+        case 12: return launch_ks_tile<KERN<12>>(12, __VA_ARGS__);             \
+        case 16: return launch_ks_tile<KERN<16>>(16, __VA_ARGS__);             \
+        case 20: return launch_ks_tile<KERN<20>>(20, __VA_ARGS__);             \
+        default: return launch_ks_tile<KERN<24>>(24, __VA_ARGS__);             \
+    }
+
+bm_status launch_extract_ks_tile(const KsKey &k, u32 cpt, uint32_t count, cudaStream_t st, const DevJob *d_jobs,
+                                 u32 steps, const u64 *ws_acc, uint64_t *d_out, u32 *status) {
+    const u32 slices = (k.n + kKskCols) / kKskCols;
+    BM_KS_TILE(k_extract_keyswitch_tile, cpt, k, count, st, d_jobs, count, slices, steps, ws_acc, d_out, status);
+}
+
+// Runs of consecutive jobs of one key long enough for the tiles take them, all
+// others the one-block-per-job kernel (neighbouring ones in one launch).
+bm_status launch_extract_ks(const KsShape &ks, const std::vector<DevJob> &dj, int device, cudaStream_t st,
+                            const DevJob *d_jobs, u32 steps, const u64 *ws_acc, uint64_t *d_out, u32 *status) {
+    const uint32_t count = (uint32_t)dj.size();
+    int sms = 0;
+    BM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
+    auto blocks = [&](uint32_t a, uint32_t b) -> bm_status {
+        if (a == b) return BM_OK;
+        const u32 S = ks_split(b - a, device);
+        if (ks.cpt == 4)
+            return launch_ks_kernel<k_extract_keyswitch<4>>(b - a, S, ks, st, d_jobs + a, steps, ws_acc, d_out);
+        return launch_ks_kernel<k_extract_keyswitch<8>>(b - a, S, ks, st, d_jobs + a, steps, ws_acc, d_out);
+    };
+    uint32_t rest = 0;
+    for (uint32_t i = 0, j; i < count; i = j) {
+        for (j = i + 1; j < count && dj[j].key == dj[i].key; j++) {}
+        const KsKey *k = nullptr;
+        for (const KsKey &x : ks.keys)
+            if (x.dev == dj[i].key) k = &x;
+        const u32 cpt = k ? ks_tile_cpt(*k, j - i, (u32)sms) : 0;
+        if (!cpt) continue;
+        bm_status s = blocks(rest, i);
+        if (s != BM_OK) return s;
+        if ((s = launch_extract_ks_tile(*k, cpt, j - i, st, d_jobs + i, steps, ws_acc, d_out, status)) !=
+            BM_OK) return s;
+        rest = j;
+    }
+    return blocks(rest, count);
 }
 
 // Every launch of one batch (the plan is already in the workspace).
@@ -655,7 +790,7 @@ bm_status launch_all(const Plan &pl, uint32_t n_persistent, const KsShape &ks, i
     if ((s = run_groups(pl, n_persistent, count, steps, d_ct_in, d_lut, ws, st, false, max_cluster, shapes)) != BM_OK)
         return s;
     if (do_ks) {
-        if ((s = launch_extract_ks(ks, count, ks_split(count, device), st, d_jobs, steps, ws_acc, d_out)) != BM_OK)
+        if ((s = launch_extract_ks(ks, pl.dj, device, st, d_jobs, steps, ws_acc, d_out, (u32 *)ws)) != BM_OK)
             return s;
     } else {
         k_copy_acc<<<count, 256, 0, st>>>(d_jobs, steps, ws_acc, d_out);
@@ -819,10 +954,17 @@ extern "C" bm_status bm_key_switch(const bm_eval_key *key, const uint64_t *d_lwe
     DeviceGuard g(key->device);
     const bm_eval_key *keys[1] = {key};
     const KsShape ks = ks_shape(keys, 1);
-    const u32 S = ks_split(count, key->device);
     cudaStream_t st = (cudaStream_t)stream;
-    if (ks.cpt == 4) return launch_ks_kernel(k_key_switch<4>, count, S, ks, st, key->d_view, d_lwe_in, d_out);
-    return launch_ks_kernel(k_key_switch<8>, count, S, ks, st, key->d_view, d_lwe_in, d_out);
+    int sms = 0;
+    BM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, key->device));
+    const KsKey &k = ks.keys[0];
+    if (const u32 cpt = ks_tile_cpt(k, count, (u32)sms)) {
+        const u32 slices = (k.n + kKskCols) / kKskCols;
+        BM_KS_TILE(k_key_switch_tile, cpt, k, count, st, key->d_view, count, slices, d_lwe_in, d_out);
+    }
+    const u32 S = ks_split(count, key->device);
+    if (ks.cpt == 4) return launch_ks_kernel<k_key_switch<4>>(count, S, ks, st, key->d_view, d_lwe_in, d_out);
+    return launch_ks_kernel<k_key_switch<8>>(count, S, ks, st, key->d_view, d_lwe_in, d_out);
 }
 
 extern "C" bm_status bm_poly_mul(const bm_eval_key *key, const uint64_t *d_a, const uint64_t *d_b,

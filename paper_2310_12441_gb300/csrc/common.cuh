@@ -17,7 +17,7 @@
 // device memory (owned by the bm_eval_key) so jobs can point at it.
 struct KeyDev {
     const u64 *bsk;    // [n][2][2 l_B][N][2], NTT domain, scaled by N^-1 (limbs, see lbits)
-    const u64 *ksk;    // [N][l_ks][B_ks - 1][n + 1]
+    const u64 *ksk;    // [N][column slices][l_ks][B_ks - 1][slice width]: ksk_slice_width
     const u64 *tw;     // forward twiddles psi^bitrev(k), k in [0, N)
     const u64 *twsh;   // their Shoup companions
     const u64 *itw;    // inverse twiddles psi^-bitrev(k)
@@ -52,6 +52,18 @@ struct DevJob {
     u64 gpre;          // u32 offset from the workspace start of the prefix sums
                        // pre[k] = (u_0 + ... + u_{k-1}) mod 2N, k in [0, m] (gS != 0)
 };
+
+// Key-switching key: the rows (j, v) of a coefficient i are stored slice by
+// slice of kKskCols columns, the last slice as wide as it has to be (even: rows
+// then begin on 16 bytes), so that one slice of a coefficient is one piece of
+// memory that a single bulk copy moves.  Row (j (B_ks - 1) + v - 1) = r, column
+// c of coefficient i: i rows ksk_pitch(n) + c0 rows + r width + c - c0, with
+// rows = l_ks (B_ks - 1), c0 = c rounded down to kKskCols.
+constexpr u32 kKskCols = 64;
+__host__ __device__ constexpr u32 ksk_pitch(u32 n) { return (n + 2) & ~1u; }
+__host__ __device__ constexpr u32 ksk_slice_width(u32 n, u32 c0) {
+    return ksk_pitch(n) - c0 < kKskCols ? ksk_pitch(n) - c0 : kKskCols;
+}
 
 // Arithmetic variants of the blind rotation, chosen per key set on the host.
 #define BR_V_QLOW1 1u   // Q = c 2^32 + 1: one-multiply q Q

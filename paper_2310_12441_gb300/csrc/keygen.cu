@@ -218,11 +218,16 @@ __device__ __forceinline__ void ksk_row(size_t row, GetA get_a, int ev, const in
     const u32 lane = threadIdx.x & 31;
     const u32 n = K.n, B1 = (1u << K.log2_Bks) - 1;
     const u64 Q = K.mq.Q;
-    u64 *o = ksk + row * (n + 1);
+    const u32 rows = K.l_ks * B1, r = (u32)(row % rows);
+    u64 *o = ksk + row / rows * rows * ksk_pitch(n);
+    auto at = [&](u32 c) -> u64 & {
+        const u32 c0 = c & ~(kKskCols - 1);
+        return o[(size_t)c0 * rows + (size_t)r * ksk_slice_width(n, c0) + c - c0];
+    };
     u64 lo = 0, hi = 0;
     for (u32 c = lane; c < n; c += 32) {
         const u64 x = get_a(c);
-        o[c] = x;
+        at(c) = x;
         const int sc = s[c];
         if (sc > 0) add128(lo, hi, x);
         else if (sc < 0) add128(lo, hi, Q - x);
@@ -238,7 +243,7 @@ __device__ __forceinline__ void ksk_row(size_t row, GetA get_a, int ev, const in
         u64 vg = reduce128(l2, h2, K.mq);
         const int zi = z[i];
         u64 msg = zi > 0 ? vg : (zi < 0 ? (vg ? Q - vg : 0) : 0);
-        o[n] = add_mod(add_mod(acc, signed_to_zq(ev, Q), Q), msg, Q);
+        at(n) = add_mod(add_mod(acc, signed_to_zq(ev, Q), Q), msg, Q);
     }
 }
 
@@ -446,7 +451,7 @@ static bm_status keygen_impl(const bm_key_params *params, const int8_t *s, const
     const size_t bsk_words = (size_t)n * 2 * 2 * lB * 2 * N;
     const u32 B1 = (1u << p.log2_Bks) - 1;
     const size_t ksk_rows = (size_t)N * p.l_ks * B1;
-    const size_t ksk_words = ksk_rows * (n + 1);
+    const size_t ksk_words = ksk_rows * ksk_pitch(n);
 
     if (cudaMalloc(&ek->d_tables, tab.size() * 8 + 8 * (size_t)N) != cudaSuccess) return BM_ENOMEM;
     if (cudaMalloc(&ek->d_bsk, bsk_words * 8) != cudaSuccess) return BM_ENOMEM;
