@@ -301,6 +301,20 @@ __device__ __forceinline__ void digit_warps(Shared &sh, unsigned char *sm, u32 c
         const u64 *cur = s.cur;
         const u64 ctk = s.ct[s.k];
         const u32 ak = (qp & (qp - 1)) == 0 ? (u32)ctk & (qp - 1) : (u32)(ctk % qp);
+        if constexpr (LOGN == 10) {
+            // A few clusters walk the key, larger than the L2, one step's rows at
+            // a time and at HBM latency: the launch's blocks bring the next
+            // step's rows to the L2, 1 KB each in turn (one job of 630 steps 17.1
+            // -> 15.7 ms, 30 jobs 16.4 -> 15.7; at N = 2048 the loads are
+            // spread over twice the work and it costs 1%).
+            if (csize > 1 && un.row == 0 && un.part == 0 && s.k + 1 < s.steps) {
+                const u32 chunks = 4 * lB * 2 * N * 8 / 1024;
+                const unsigned char *next = (const unsigned char *)(K->bsk + (size_t)(s.k + 1) * 4 * lB * 2 * N);
+                for (u32 ch = blockIdx.x + dt * gridDim.x; ch < chunks; ch += kD * gridDim.x)
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(next + (size_t)ch * 1024), "r"(1024u)
+                                 : "memory");
+            }
+        }
         const u32 dmask = ((1u << log2B) - 1) * 0x10001u;
         const u32 dcen = (0x6400u | (1u << (log2B - 1))) * 0x10001u;     // fp16 1024 + 2^(log2 B - 1), twice
         u32 got = 0, c = 0;  // tiles taken, digit polynomials done

@@ -8,7 +8,8 @@
 // spilled about 9.6 KB per thread.  Per class, the kernel spills at most a
 // few bytes.  The host launches the classes concurrently (forked streams,
 // longest class first), so the blocks of a later class take over each SM as
-// the earlier class runs out of jobs.
+// the earlier class runs out of jobs.  Classes of keys with tensor-core stages
+// run br_tc.cu's kernel at shape 1, which pulls jobs the same way.
 #include "br_launch.cuh"
 
 namespace {
