@@ -108,7 +108,7 @@ inline u32 choose_variant(const bm_key_params &p) {
     // The tensor-core stages (br_tc.cuh): digits of at most 10 bits (9 at N =
     // 1024), the digits of two (sign, component) pairs (N = 1024) or one (N =
     // 2048) in whole half batches, within the shared memory beside the weights.
-    // Every such key gains (one bootstrap at N = 1024: 18.6 ms without, 15.4 with
+    // Every such key gains (one bootstrap at N = 1024: 18.7 ms without, 15.9 with
     // them; full blocks as in br_tc.cuh), so no size is left to the other form.
     const bool tc1 = p.Q < (1ull << 54) && p.log2_B <= 9;
     if ((v & BR_V_QLOW1) && p.l_B <= 6 && p.l_B % 2 == 0 && p.log2_B <= 10 &&
