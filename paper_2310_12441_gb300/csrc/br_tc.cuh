@@ -36,6 +36,15 @@
 // A block works on two jobs in turn, one CMux step of each at a time, so the
 // inverse transforms and digits at a job's step boundary overlap the other
 // job's transforms; blocks take further jobs from a counter.
+//
+// What bounds it: the 32-bit multiplier pipe (recombination, three or four
+// remaining stages, multiply-accumulate, inverse transforms), 68% busy with two
+// jobs in every block (61% with one) against 59% (50%) of the issue slots and
+// 10% of the tensor pipe; at N = 2048 the transform warps' integer instructions.
+// Per row of one CMux step and SM, blocks full: N = 1024, Q < 2^54: 24.9 us with
+// all stages in the CUDA cores (br_job), 16.7 us here; N = 2048, Q < 2^60: 64.2
+// and 56.3 us.  1000 bootstraps at N = 1024 with m = 4: 444 and 313 ms; 200 at
+// N = 2048 with m = 8: 579 and 511 ms.
 #pragma once
 #include "blind_rotate.cuh"
 #include <cuda_fp16.h>
