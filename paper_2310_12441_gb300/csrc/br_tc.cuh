@@ -47,7 +47,7 @@
 // N = 2048 with m = 8: 579 and 511 ms.
 #pragma once
 #include "blind_rotate.cuh"
-#include <cuda_fp16.h>
+#include "tc_tables.cuh"
 
 namespace brt {
 
@@ -55,14 +55,6 @@ constexpr u32 kT = 256, kM = 256;            // transform and product threads
 constexpr u32 kD = 96;                       // digit threads
 constexpr u32 kThreads = kT + kM + 32 + kD;  // + the issuing warp
 constexpr u32 kTile = 16384;                 // B bytes of one batch (8 half-column tiles of 2 KB)
-
-// Tensor-core configurations (signed limbs of the weights): TC1 for Q < 2^54
-// and log2 B <= 9, TC2 for Q < 2^60 and log2 B <= 10.
-template <int TC>
-struct Limbs {
-    static constexpr int NL = TC == 1 ? 5 : 6;
-    static constexpr int R = TC == 1 ? 11 : 10;
-};
 
 template <int LOGN, int TC>
 struct Cfg {
@@ -410,35 +402,6 @@ __device__ __forceinline__ void digit_warps(Shared &sh, unsigned char *sm, u32 c
     }
 }
 
-// Limbs of one value -> E or O modulo Q: sum_l o_l 2^(R l) + cst - q Q with
-// the quotient q of the value's top bits (at most 2 below the true one), the
-// sum modulo 2^64.  cst carries the centring constant and a multiple of Q
-// above every negative value.
-template <int TC>
-__device__ __forceinline__ u64 recombine(const u32 (&f)[Limbs<TC>::NL], u64 cst, u32 t0, u32 mq, u32 c) {
-    constexpr int R = Limbs<TC>::R, NL = Limbs<TC>::NL;
-    int32_t o[NL];
-#pragma unroll
-    for (int l = 0; l < NL; l++) o[l] = __float2int_rn(__uint_as_float(f[l]));
-    // value modulo 2^64
-    auto plus = [](u64 t, int32_t v, int32_t k) {
-        u64 r;
-        asm("{\n\t.reg .u64 p;\n\tmul.wide.s32 p, %2, %3;\n\tadd.u64 %0, %1, p;\n\t}" : "=l"(r) : "l"(t), "r"(v), "r"(k));
-        return r;
-    };
-    u64 t = plus(plus(cst, o[1], 1 << R), o[2], 1 << (2 * R));
-    if constexpr (NL == 6) t = plus(t, o[3], 1 << (3 * R));
-    t = add64c(t, (u64)(int64_t)o[0]);
-    u32 hi = (u32)(t >> 32) + ((u32)o[NL - 1] << ((NL - 1) * R - 32));
-    hi += (u32)o[NL - 2] << ((NL - 2) * R - 32);
-    if constexpr (NL == 5) static_assert((NL - 2) * R >= 32, "high limbs");
-    // quotient from the top limbs, in units of 2^((NL - 1) R - 4)
-    const u32 v = ((u32)o[NL - 1] << 4) + (u32)(o[NL - 2] >> (R - 4)) + t0;
-    const u32 q = __umulhi(v, mq);
-    hi -= q * c;
-    return sub64c(((u64)hi << 32) | (u32)t, q);
-}
-
 // v minus 8Q when v >= 2^63 (Q < 2^60: the result is below 2^63).
 __device__ __forceinline__ u64 csub8q(u64 v, u64 eightQ) {
     const u64 mask = (u64)((int64_t)v >> 63);
@@ -447,8 +410,8 @@ __device__ __forceinline__ u64 csub8q(u64 v, u64 eightQ) {
 
 // Last stages of one class in registers: V values, twiddles tw(t) (t = 0 ..
 // V - 2 in stage order).  LAZY: no corrections, every stage but the last widens
-// the range by 4Q to both sides (the last by 8Q upwards); else (Q < 2^60,
-// values start below 6.3Q) two stages without correction (14.3Q), one
+// the range by 4Q to both sides (the last by 4Q upwards); else (Q < 2^60,
+// values start below 6.34Q) two stages without correction (14.34Q), one
 // subtraction of 8Q from values above 2^63, two more stages: below 2^63 + 8Q.
 template <int V, bool LAZY, class Tw>
 __device__ __forceinline__ void class_stages(u64 (&x)[V], Tw tw, u32 c, u64 fourQ) {
@@ -612,7 +575,8 @@ __device__ __forceinline__ void transform_warps(Shared &sh, unsigned char *sm, u
                                 a[l] = f[jj & 1][l][j];
                                 o[l] = f[jj & 1][NL + l][j];
                             }
-                            const u64 E = recombine<TC>(a, cE, t0, tcm, cq), O = recombine<TC>(o, cO, t0, tcm, cq);
+                            const u64 E = recombine<TC, LAZY>(a, cE, t0, tcm, cq);
+                            const u64 O = recombine<TC, LAZY>(o, cO, t0, tcm, cq);
                             y0[jj * 2 + j] = add64c(E, O);      // class 2p
                             y1[jj * 2 + j] = sub64c(E, O);      // class 2p + 1
                         }

@@ -15,11 +15,10 @@
 #include <new>
 #include <vector>
 
-#include <cuda_fp16.h>
-
 #include "common.cuh"
 #include "ntt.cuh"
 #include "philox.cuh"
+#include "tc_tables.cuh"
 
 typedef unsigned __int128 u128;
 
@@ -300,82 +299,6 @@ static void fill_keydev_constants(KeyDev &K, const bm_key_params &p, u32 logN, u
     (void)psi;
 }
 
-// Tables of the tensor-core transform stages (br_tc.cuh) for a key with a
-// BR_V_TC* flag: fp16 limbs of the weights w_p^(2i), w_p^(2i + 1) (centred
-// modulo Q, signed limbs of R bits, K-major 8x16-byte core matrices), the
-// additive constants of the E and O sums, the twiddle pairs of stages 7 and
-// up, [stage position][class parity][class / 2], and the inverse pairs in the
-// order of ntr::inv_twiddle_slot for radix 8.
-static std::vector<unsigned char> tc_tables(const bm_key_params &p, u32 variant, const std::vector<u64> &tab,
-                                            KeyDev &K) {
-    const u32 NL = (variant & BR_V_TC1) ? 5 : 6, R = (variant & BR_V_TC1) ? 11 : 10, N = p.N;
-    const u64 Q = p.Q;
-    const u32 nt = N / 128 - 1;
-    std::vector<unsigned char> out(NL * 16384 + 1024 + (size_t)nt * 2048 + (size_t)N * 16);
-    // a multiple of Q above every |sum|: sums stay within 64 2^(log2 B - 1) 2^(R - 1) per limb
-    const u32 sbits = 6 + p.log2_B - 1 + R - 1 + (NL - 1) * R;
-    const u128 off = ((((u128)1 << sbits) + ((u128)1 << (sbits - 4))) / Q + 1) * Q;
-    const u32 unit = (NL - 1) * R - 4;
-    // 600 units cover the limbs the quotient estimate leaves out
-    K.tc_t0 = (u32)(off >> unit) - 600u;
-    K.tc_m = (u32)(((u128)1 << (unit + 32)) / Q);
-    // limb radices of the multiply-accumulate with their Shoup companions
-    const u32 lb = br_qlow1_limb((variant & BR_V_LAZY) != 0);
-    K.tc_b1 = (1ull << lb) % Q;
-    K.tc_b1s = shoup_of(K.tc_b1, Q);
-    K.tc_b2 = (1ull << (2 * lb)) % Q;
-    K.tc_b2s = shoup_of(K.tc_b2, Q);
-    // (v >> 32) / (c + 1) with c = Q >> 32, 2^tc_fsh <= c < 2^(tc_fsh + 1)
-    const u64 c1 = (Q >> 32) + 1;
-    K.tc_fsh = 0;
-    while ((2ull << K.tc_fsh) < c1) K.tc_fsh++;
-    K.tc_fs = (u32)(((u128)1 << (32 + K.tc_fsh)) / c1);
-    for (u32 c = 0; c < 64; c++) {
-        const u64 w = tab[64 + c], w2 = host_mulmod(w, w, Q);
-        u64 f[2] = {1 % Q, w};
-        u128 sum[2] = {0, 0};
-        for (u32 i = 0; i < 64; i++) {
-            for (u32 e = 0; e < 2; e++) {
-                sum[e] += f[e];
-                int64_t v = f[e] > Q / 2 ? (int64_t)f[e] - (int64_t)Q : (int64_t)f[e];
-                for (u32 l = 0; l < NL; l++) {
-                    int64_t r = v;
-                    if (l + 1 < NL) {
-                        r = ((v + (1 << (R - 1))) & ((1 << R) - 1)) - (1 << (R - 1));
-                        v = (v - r) >> R;
-                    }
-                    const __half h = __float2half((float)r);
-                    memcpy(&out[(e * NL + l) * 8192 + (c / 8) * 1024 + (i / 8) * 128 + (c % 8) * 16 + (i % 8) * 2], &h, 2);
-                }
-                f[e] = host_mulmod(f[e], w2, Q);
-            }
-        }
-        for (u32 e = 0; e < 2; e++) {
-            u64 cst = host_mulmod((u64)(sum[e] % Q), (1ull << (p.log2_B - 1)) % Q, Q);
-            // E in [2Q, 4.3Q), O in [-2Q, 0.3Q); lazy keys start 4Q higher per
-            // remaining stage but the last
-            const u64 up = (variant & BR_V_LAZY) ? 4 * (u64)(K.logN - 8) : 0;
-            cst += (u64)off + (e == 0 ? (2 + up) * Q : 0 - 2 * Q);
-            memcpy(&out[NL * 16384 + e * 512 + c * 8], &cst, 8);
-        }
-    }
-    u32 pos = 0;
-    for (u32 s = 7; (1u << s) < N; s++)
-        for (u32 g = 0; g < (1u << (s - 7)); g++, pos++)
-            for (u32 k = 0; k < 128; k++)
-                memcpy(&out[NL * 16384 + 1024 + pos * 2048 + ((k & 1) * 64 + k / 2) * 16],
-                       &tab[4 * (size_t)N + 2 * ((1u << s) + (k << (s - 7)) + g)], 16);
-    for (u32 i = 1; i < N; i++) {
-        u32 s = 0;
-        while ((2u << s) <= i) s++;
-        const u32 q = (K.logN - 1 - s) / 3, F = q < (K.logN + 2) / 3 - 1 ? 3 * q : K.logN - 3, sh = K.logN - 3 - F;
-        const u32 r = i - (1u << s), j = r >> sh, high = r & ((1u << sh) - 1);
-        memcpy(&out[NL * 16384 + 1024 + (size_t)nt * 2048 + (size_t)i * 16],
-               &tab[6 * (size_t)N + 2 * ((1u << s) + ((high << (s - sh)) | j))], 16);
-    }
-    return out;
-}
-
 static u64 find_psi(u64 Q, u32 N) {
     for (u64 g = 2; g < 1000000; g++) {
         u64 psi = host_powmod(g, (Q - 1) / (2ull * N), Q);
@@ -475,7 +398,7 @@ static bm_status keygen_impl(const bm_key_params *params, const int8_t *s, const
     K.tc_b1 = K.tc_b1s = K.tc_b2 = K.tc_b2s = 0;
     const u32 variant = choose_variant(p);
     if (variant & (BR_V_TC1 | BR_V_TC2)) {
-        const std::vector<unsigned char> tct = tc_tables(p, variant, tab, K);
+        const std::vector<unsigned char> tct = brt::tc_tables(p, variant, tab, K);
         if (cudaMalloc(&ek->d_tc, tct.size()) != cudaSuccess) return BM_ENOMEM;
         ek->bytes += tct.size();
         BM_CUDA_TRY(cudaMemcpy(ek->d_tc, tct.data(), tct.size(), cudaMemcpyHostToDevice));
