@@ -132,7 +132,48 @@ __device__ __forceinline__ void tmem_st16(u32 addr, const u32 (&r)[16]) {
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// Barrier of the product warps.
 __device__ __forceinline__ void bar_m() { asm volatile("bar.sync 5, 256;" ::: "memory"); }
+
+// Waits of a whole warp for the phase of `bar` with this parity (acquire, CLUSTER:
+// from the blocks of the cluster).  Bounded: a warp that polled `polls` times
+// (each poll may suspend it for a while) sets BM_ETIMEDOUT in the status word
+// and `dead` for the block, which every wait that goes on polling looks at.
+// False, for the whole warp alike: the block has given up.  (No correct launch
+// has such a wait.)  Transform, digit and issuing warps then leave at once;
+// product warps share barriers, so they go on without waiting, on words that
+// need not be what they should be, to the step's end and leave there together
+// (bar_or), before another job's state can take the slot's place.
+constexpr u32 kPolls = 1u << 24;
+template <bool CLUSTER = false>
+__device__ __forceinline__ bool poll(u64 *bar, u32 parity) {
+    u32 ok;
+    if constexpr (CLUSTER)
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok)
+                     : "r"(smem_u32(bar)), "r"(parity)
+                     : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok)
+                     : "r"(smem_u32(bar)), "r"(parity)
+                     : "memory");
+    return __all_sync(0xffffffffu, ok);
+}
+template <bool CLUSTER = false>
+[[nodiscard]] __device__ __forceinline__ bool wait(u64 *bar, u32 parity, u32 *dead, u32 *status, u32 polls = kPolls) {
+    for (u32 it = 0; !poll<CLUSTER>(bar, parity); it++) {
+        if (it == polls) {
+            set_status(status, BM_ETIMEDOUT);
+            *(volatile u32 *)dead = 1;
+            return false;
+        }
+        if (it % 32 == 31 && __any_sync(0xffffffffu, *(volatile u32 *)dead)) return false;
+    }
+    return true;
+}
 
 // Register split of the 640 threads launched with 96 each: per thread of four
 // warps 2 x 88 + 2 x 112 + 80 = 480 = 5 x 96, exactly what the block holds.
@@ -166,11 +207,24 @@ struct Shared {
     u64 tfull, tempty;      // a batch's accumulators complete / read (transform warps)
     u64 xfull[2], xempty[2];    // a stage's polynomials stored / multiplied
     u64 cbar;               // cluster barrier of the product warps
+    u64 drain;              // every product complete
+    u32 dead;               // a wait of this block has given up: every role leaves
     u32 tmem;
     u32 next;               // a job index taken from the counter
     u32 taken;              // jobs this block has started
     int bad;
 };
+
+// bar_m that says, to all product warps alike, whether the block has given up.
+__device__ __forceinline__ bool bar_or(Shared &sh) {
+    u32 r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 5, 256, p;\n\t"
+                 "selp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(r)
+                 : "r"(*(volatile u32 *)&sh.dead)
+                 : "memory");
+    return r != 0;
+}
 
 __device__ __forceinline__ void open(Shared &sh, u32 csize) {
     if (threadIdx.x == 0) {
@@ -186,6 +240,8 @@ __device__ __forceinline__ void open(Shared &sh, u32 csize) {
             mbar_init(&sh.xempty[i], kM / 32);
         }
         mbar_init(&sh.cbar, csize * (kM / 32));
+        mbar_init(&sh.drain, 1);
+        sh.dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (threadIdx.x / 32 == (kT + kM) / 32) {
@@ -208,8 +264,8 @@ __device__ __forceinline__ void close(Shared &sh, u32 csize) {
 }
 
 // One step's barrier over the product warps of every block of a cluster
-// (global writes before it are visible after it).
-__device__ __forceinline__ void cluster_bar_m(Shared &sh, u32 csize, u32 &parity, u32 *status) {
+// (global writes before it are visible after it); false as wait().
+[[nodiscard]] __device__ __forceinline__ bool cluster_bar_m(Shared &sh, u32 csize, u32 &parity, u32 *status) {
     __threadfence();
     __syncwarp();
     if (threadIdx.x % 32 == 0) {
@@ -220,21 +276,10 @@ __device__ __forceinline__ void cluster_bar_m(Shared &sh, u32 csize, u32 &parity
             asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
         }
     }
-    for (u32 it = 0;; it++) {
-        u32 ok;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok)
-                     : "r"(smem_u32(&sh.cbar)), "r"(parity)
-                     : "memory");
-        if (ok) break;
-        if (it == (1u << 24)) {
-            set_status(status, BM_ETIMEDOUT);
-            break;
-        }
-    }
+    const bool ok = wait<true>(&sh.cbar, parity, &sh.dead, status);
     parity ^= 1;
     __threadfence();
+    return ok;
 }
 
 // The issuing warp: per unit its batches; per batch A E / O x limbs x two
@@ -246,12 +291,13 @@ __device__ __forceinline__ void issuer(Shared &sh, unsigned char *sm, u32 *statu
     const u64 da = smem_desc(sa, 128, 1024);
     u32 pb = 0, pe = 1;      // (tempty: the first wait passes, as if a batch had been read)
     for (u32 u = 0;; u++) {
-        mbar_wait(&sh.post[u & 1], (u >> 1) & 1, status);
+        bool ok = wait(&sh.post[u & 1], (u >> 1) & 1, &sh.dead, status);
         const u32 ncomb = *(volatile u32 *)&sh.unit[u & 3].ncomb;
-        for (u32 b = 0; b * C::CB < ncomb; b++) {
-            mbar_wait(&sh.bfull[b], (pb >> b) & 1, status);
+        for (u32 b = 0; ok && b * C::CB < ncomb; b++) {
+            // (tempty: the previous batch's accumulators have been read)
+            ok = wait(&sh.bfull[b], (pb >> b) & 1, &sh.dead, status) && wait(&sh.tempty, pe, &sh.dead, status);
+            if (!ok) break;
             pb ^= 1u << b;
-            mbar_wait(&sh.tempty, pe, status);     // the previous batch's accumulators have been read
             pe ^= 1;
             fence_after();
             if (elect_one()) {
@@ -275,11 +321,16 @@ __device__ __forceinline__ void issuer(Shared &sh, unsigned char *sm, u32 *statu
             }
             __syncwarp();
         }
+        if (!ok) break;
         if (ncomb == 0) {      // wakes the transform warps, which leave too
             if (elect_one()) mbar_arrive(&sh.tfull);
             break;
         }
     }
+    // no product may be outstanding when the block ends (none is, unless it gave up)
+    if (elect_one()) mma_commit(&sh.drain);
+    __syncwarp();
+    for (u32 it = 0; it < kPolls && !poll(&sh.drain, 0); it++) {}
 }
 
 // Digit warps: for every unit and pair the differences D = P(c) ACC - ACC of
@@ -292,7 +343,7 @@ __device__ __forceinline__ void digit_warps(Shared &sh, unsigned char *sm, u32 c
     const u32 dt = threadIdx.x - (kT + kM + 32), lane = dt % 32;
     u32 pe = 7;              // bempty parities (first waits pass)
     for (u32 u = 0;; u++) {
-        mbar_wait(&sh.post[u & 1], (u >> 1) & 1, status);
+        if (!wait(&sh.post[u & 1], (u >> 1) & 1, &sh.dead, status)) return;
         const Unit un = *(const Unit *)&sh.unit[u & 3];
         if (un.ncomb == 0) break;
         const KeyDev *K = sh.key;
@@ -323,7 +374,7 @@ __device__ __forceinline__ void digit_warps(Shared &sh, unsigned char *sm, u32 c
         for (u32 pr = 0; pr < (u32)C::PAIRS; pr++) {
             for (u32 b = c / C::CB; b <= (c + lB - 1) / C::CB; b++)
                 if (!((got >> b) & 1)) {
-                    mbar_wait(&sh.bempty[b], (pe >> b) & 1, status);
+                    if (!wait(&sh.bempty[b], (pe >> b) & 1, &sh.dead, status)) return;
                     pe ^= 1u << b;
                     got |= 1u << b;
                 }
@@ -527,7 +578,7 @@ __device__ __forceinline__ void transform_warps(Shared &sh, unsigned char *sm, u
     const ulonglong2 *tws = (const ulonglong2 *)(sm + C::TW_OFF);
     u32 pf = 0, px = 3;      // parities; px: one bit per stage (first waits pass)
     for (u32 u = 0;; u++) {
-        mbar_wait(&sh.tfull, pf, status);     // the unit's first batch (or the end)
+        if (!wait(&sh.tfull, pf, &sh.dead, status)) return;     // the unit's first batch (or the end)
         const u32 ncu = *(volatile u32 *)&sh.unit[u & 3].ncomb;
         if (ncu == 0) break;
         if (*(volatile u32 *)&sh.unit[u & 3].newkey) {
@@ -547,7 +598,7 @@ __device__ __forceinline__ void transform_warps(Shared &sh, unsigned char *sm, u
         for (u32 c0 = 0; c0 < ncu; c0 += C::CB) {
             const u32 nc = ncu - c0 < (u32)C::CB ? ncu - c0 : (u32)C::CB;
             const u32 rounds = (nc + C::RC - 1) / C::RC;
-            if (c0) mbar_wait(&sh.tfull, pf, status);
+            if (c0 && !wait(&sh.tfull, pf, &sh.dead, status)) return;
             pf ^= 1;
             fence_after();
 #pragma unroll 1
@@ -599,7 +650,7 @@ __device__ __forceinline__ void transform_warps(Shared &sh, unsigned char *sm, u
                 if constexpr (LOGN == 10) {
                     class_stages<8, LAZY>(y0, [&](int i) { return tws[i * 128 + p]; }, cq, fourQ);
                     class_stages<8, LAZY>(y1, [&](int i) { return tws[i * 128 + 64 + p]; }, cq, fourQ);
-                    mbar_wait(&sh.xempty[r], (px >> r) & 1, status);
+                    if (!wait(&sh.xempty[r], (px >> r) & 1, &sh.dead, status)) return;
                     u64 *xo = xs + (size_t)(2 * w + half) * N + p * 16;
 #pragma unroll
                     for (u32 i = 0; i < 4; i++) {
@@ -622,7 +673,7 @@ __device__ __forceinline__ void transform_warps(Shared &sh, unsigned char *sm, u
                     class_stages<16, LAZY>(x, [&](int i) {
                         return i < C::NTS ? tws[i * 128 + half * 64 + p] : __ldg(tw + i * 128 + half * 64 + p);
                     }, cq, fourQ);
-                    mbar_wait(&sh.xempty[r], (px >> r) & 1, status);
+                    if (!wait(&sh.xempty[r], (px >> r) & 1, &sh.dead, status)) return;
                     u64 *xo = xs + (size_t)w * N + (2 * p + half) * 16;
 #pragma unroll
                     for (u32 i = 0; i < 8; i++)
@@ -797,7 +848,8 @@ struct Product {
                 const u64 *kr = kp + (size_t)(c0 + r * C::RC) * 2 * N;
                 const bool last = c0 + (r + 1) * C::RC >= ncu;
                 const bool first = part == 0 && c0 == 0 && r == 0;
-                mbar_wait(&sh.xfull[r], (px >> r) & 1, status);
+                // (given up: on to the step's end)
+                (void)wait(&sh.xfull[r], (px >> r) & 1, &sh.dead, status);
                 px ^= 1u << r;
 #pragma unroll
                 for (int h = 0; h < C::PH; h++) {
@@ -875,8 +927,9 @@ struct Product {
             }
     }
 
-    // Row sums -> inverse transforms -> accumulator update of row `row`.
-    __device__ __forceinline__ void finish_row(const Slot &s, u32 row) {
+    // Row sums -> inverse transforms -> accumulator update of row `row`; false
+    // when the block has given up.
+    __device__ __forceinline__ bool finish_row(const Slot &s, u32 row) {
         constexpr int RB = 3, T = N / 8, PP = 2048 / N;         // polynomials at a time
         constexpr int NPH = (LOGN + RB - 1) / RB;
         const ModQ mq = K->mq;
@@ -946,6 +999,7 @@ struct Product {
             }
             bar_m();     // the region is read: the next sums may be written
         }
+        return true;
     }
 };
 
@@ -967,6 +1021,7 @@ __device__ __forceinline__ void product_warps(Shared &sh, unsigned char *sm, con
     bar_m();
     // a job waiting for its slot (its key is not the one loaded), or none
     u32 wait0 = blockIdx.x / csize, wait1 = csize > 1 ? count : blockIdx.x + gridDim.x;
+    bool dead = false;     // the block has given up
     // Fills an idle slot: the waiting job, or the next of the counter.
     auto fill = [&](int s) {
         u32 &w = s ? wait1 : wait0;
@@ -993,16 +1048,20 @@ __device__ __forceinline__ void product_warps(Shared &sh, unsigned char *sm, con
                 pr.load_key(key);
             }
             pr.start(s, w);
-            if (csize > 1) cluster_bar_m(sh, csize, pr.pcl, status);
+            if (csize > 1) {
+                (void)cluster_bar_m(sh, csize, pr.pcl, status);
+                dead = bar_or(sh);
+            }
             w = csize > 1 ? count : 0xffffffffu;
         }
     };
     fill(0);
     fill(1);
     u32 cs = sl[0].on ? 0 : 1;
-    if (sl[cs].on && sl[cs].mr == 0) {
+    if (dead) {
+    } else if (sl[cs].on && sl[cs].mr == 0) {
         // a cluster block without rows: only the barriers
-        for (u32 k = 0; k < sl[cs].steps; k++) cluster_bar_m(sh, csize, pr.pcl, status);
+        for (u32 k = 0; k < sl[cs].steps && cluster_bar_m(sh, csize, pr.pcl, status); k++) {}
     } else if (sl[cs].on) {
         u32 row = 0, h = 0;
         pr.post(cs, 0, 0);
@@ -1022,9 +1081,9 @@ __device__ __forceinline__ void product_warps(Shared &sh, unsigned char *sm, con
             if (ahead) pr.post(ns, nrow, nh);
             pr.products(sl[cs], h);
             if (h + 1 == units) {
-                pr.finish_row(sl[cs], row);
+                if (!pr.finish_row(sl[cs], row)) break;
                 if (!same) {
-                    if (csize > 1) cluster_bar_m(sh, csize, pr.pcl, status);
+                    if (csize > 1) (void)cluster_bar_m(sh, csize, pr.pcl, status);
                     if (pr.mtid == 0) {
                         Slot &s = sl[cs];
                         u64 *tmp = s.cur;
@@ -1032,7 +1091,7 @@ __device__ __forceinline__ void product_warps(Shared &sh, unsigned char *sm, con
                         s.nxt = tmp;
                         if (++s.k == s.steps) s.on = 0;
                     }
-                    bar_m();
+                    if (bar_or(sh)) break;
                     if (!sl[cs].on) {
                         fill(cs);
                         fill(cs ^ 1);
