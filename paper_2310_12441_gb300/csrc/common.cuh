@@ -145,10 +145,14 @@ inline void limb_plan(const bm_key_params &p, u32 variant, u32 &lbits, u32 &fold
 }
 
 // Workspace header: [0] status word, [1 + c] job counter of persistent class c,
-// [BM_WS_GROUP_WORD] job counter of a grouped launch.
+// [BM_WS_GROUP_WORD] job counter of a grouped launch.  Ring degrees 1024, 2048
+// and 4096 have 5, 7 and 4 variants (choose_variant), so a batch has at most 16
+// persistent classes.
+#define BM_WS_HEADER 256
 #define BM_WS_COUNTER_WORD 1
-#define BM_MAX_CLASSES 15
-#define BM_WS_GROUP_WORD 16
+#define BM_MAX_CLASSES 16
+#define BM_WS_GROUP_WORD (BM_WS_COUNTER_WORD + BM_MAX_CLASSES)
+static_assert(4 * (BM_WS_GROUP_WORD + 1) <= BM_WS_HEADER, "words of the workspace header");
 
 // Host-side evaluation key.
 struct bm_eval_key {
@@ -177,9 +181,6 @@ struct bm_secret_key {
             return BM_ECUDA;                                                \
         }                                                                   \
     } while (0)
-
-// Workspace header: the device status word sits at offset 0.
-#define BM_WS_HEADER 256
 
 // Persistent blind rotation of one class of jobs (same ring degree 1024..4096
 // and arithmetic variant; persistent.cu): one block per SM pulls the class's
