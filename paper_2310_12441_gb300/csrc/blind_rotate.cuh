@@ -276,7 +276,7 @@ struct Cfg {
 // row sums go to the job's sum buffer; after the last row the 2m sums are
 // inverse-transformed (P per batch) and added to the rows of the next ACC
 // buffer.
-template <int LOGN, int THREADS, int RB, bool LAZY, bool SMALL0, bool QLOW1, int BLK = 1>
+template <int LOGN, int THREADS, int RB, bool LAZY, bool SMALL0, bool QLOW1, int BLK = 1, bool WIDE = false>
 __device__ __forceinline__ void br_job(const DevJob &J, u32 steps_limit, const u64 *__restrict__ ct_in,
                                        const u32 *__restrict__ luts, u64 *ws, u32 *status, u64 *sm) {
     using C = Cfg<LOGN, THREADS, RB, BLK>;
@@ -284,7 +284,7 @@ __device__ __forceinline__ void br_job(const DevJob &J, u32 steps_limit, const u
     constexpr int N = C::N, G = C::G, CPB = C::CPB;
     const KeyDev *K = J.key;
     // (keys of the Q = c 2^32 + 1 kernels have limbs of a fixed width)
-    constexpr u32 LB = br_qlow1_limb(LAZY);
+    constexpr u32 LB = br_qlow1_limb((LAZY ? BR_V_LAZY : 0) | (WIDE ? BR_V_WIDE : 0));
     const u32 lbits = QLOW1 ? LB : J.lbits;
     const bool fold_each = J.fold_each != 0;
     const u32 m = J.m, t = J.t, lB = K->l_B, log2B = K->log2_B, n = K->n;

@@ -496,9 +496,7 @@ bm_status make_plan(const bm_eval_key *const *keys, const bm_job *jobs, uint32_t
 
 // Kernel shape per ring degree (log2 N = 8..13) used by launches that do
 // not carry their own: the autotuner's choice once it has run, else the
-// measured best of each degree (radix 8 with 1024 threads for N = 1024 ..
-// 8192; radix 16 with 512 threads below).
-constexpr u32 kDefaultShape[14] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1};
+// default of the degree.
 std::atomic<u32> g_shape[14] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1};
 
 struct Shapes {
@@ -1252,7 +1250,7 @@ extern "C" bm_status bm_kernel_shape_info(uint32_t shape, uint32_t N, uint32_t *
 extern "C" bm_status bm_set_kernel_shape(uint32_t N, uint32_t shape) {
     if (N < 256 || N > BM_MAX_N_BLOCK || (N & (N - 1))) return BM_EINVAL;
     const u32 l = log2u(N);
-    if (shape == BM_SHAPE_DEFAULT) shape = kDefaultShape[l];
+    if (shape == BM_SHAPE_DEFAULT) shape = (uint32_t)br_default_shape((int)l);
     if (bm_kernel_shape_info(shape, N, nullptr, nullptr, nullptr) != BM_OK) return BM_EINVAL;
     g_shape[l].store(shape);
     return BM_OK;

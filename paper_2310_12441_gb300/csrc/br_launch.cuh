@@ -23,6 +23,9 @@ __host__ __device__ constexpr BrShape br_shape(int sh) {
          : sh == 4 ? BrShape{3, 512, 1}
                    : BrShape{4, 512, 1};
 }
+// The measured best of each ring degree: radix 8 with 1024 threads for N = 1024
+// .. 8192; radix 16 with 512 threads below.
+__host__ __device__ constexpr int br_default_shape(int logn) { return logn >= 10 ? 1 : 0; }
 __host__ __device__ constexpr bool br_shape_fits(int logn, int sh) {
     const BrShape b = br_shape(sh);
     const int T = (1 << logn) >> b.rb;
@@ -31,13 +34,13 @@ __host__ __device__ constexpr bool br_shape_fits(int logn, int sh) {
     return smem <= 226 * 1024 && (smem + 1024) * b.blocks <= 228 * 1024;
 }
 
-template <int LOGN, int SH, bool LAZY, bool SMALL0, bool QLOW1>
+template <int LOGN, int SH, bool LAZY, bool SMALL0, bool QLOW1, bool WIDE>
 __global__ void __launch_bounds__(br_shape(SH).threads, br_shape(SH).blocks)
     k_blind_rotate(const DevJob *__restrict__ jobs, u32 steps_limit, const u64 *__restrict__ ct_in,
                    const u32 *__restrict__ luts, u64 *ws, u32 *status) {
     extern __shared__ __align__(16) u64 sm[];
     // a cluster of blocks shares one job (rows split); plain launches: 1 block
-    brk::br_job<LOGN, br_shape(SH).threads, br_shape(SH).rb, LAZY, SMALL0, QLOW1, br_shape(SH).blocks>(
+    brk::br_job<LOGN, br_shape(SH).threads, br_shape(SH).rb, LAZY, SMALL0, QLOW1, br_shape(SH).blocks, WIDE>(
         jobs[blockIdx.x / cluster_size()], steps_limit, ct_in, luts, ws, status, sm);
 }
 
@@ -108,13 +111,13 @@ u32 pick_cluster(K kern, u32 threads, size_t smem, u32 cnt, u32 mmax, u32 max_cl
 
 // dry: only set the kernel's attributes and occupancy (done before a
 // CUDA-graph capture).
-template <int LOGN, int SH, bool LAZY, bool SMALL0, bool QLOW1>
+template <int LOGN, int SH, bool LAZY, bool SMALL0, bool QLOW1, bool WIDE = false>
 bm_status launch_br_v(const DevJob *jobs, uint32_t cnt, u32 mmax, u32 max_cluster, u32 steps,
                       const uint64_t *ct_in, const uint32_t *lut, u64 *ws_acc, u32 *status, cudaStream_t st,
                       bool dry) {
     using C = brk::Cfg<LOGN, br_shape(SH).threads, br_shape(SH).rb, br_shape(SH).blocks>;
     static std::atomic<uint64_t> attr_done{0};
-    auto kern = k_blind_rotate<LOGN, SH, LAZY, SMALL0, QLOW1>;
+    auto kern = k_blind_rotate<LOGN, SH, LAZY, SMALL0, QLOW1, WIDE>;
     bm_status s = ensure_smem(kern, C::SMEM, attr_done);
     if (s != BM_OK) return s;
     const u32 S = max_cluster > 1 ? pick_cluster(kern, C::kThreads, C::SMEM, cnt, mmax, max_cluster) : 1;
@@ -170,6 +173,9 @@ bm_status launch_br(u32 variant, u32 shape, const DevJob *jobs, uint32_t cnt, u3
 #define BM_LAUNCH(LZ, S0, QL) \
     return launch_shape<LOGN, LZ, S0, QL>(shape, jobs, cnt, mmax, max_cluster, steps, ct_in, lut, ws_acc, status, st, dry)
     switch (variant & BR_V_ARITH) {
+        case BR_V_LAZY | BR_V_QLOW1 | BR_V_WIDE:     // (a band of 6% in Q: the default shape only)
+            return launch_br_v<LOGN, br_default_shape(LOGN), true, true, true, true>(jobs, cnt, mmax, max_cluster, steps,
+                                                                                    ct_in, lut, ws_acc, status, st, dry);
         case BR_V_LAZY | BR_V_QLOW1: BM_LAUNCH(true, true, true);
         case BR_V_LAZY: BM_LAUNCH(true, true, false);
         case BR_V_QLOW1: BM_LAUNCH(false, true, true);
@@ -180,6 +186,7 @@ bm_status launch_br(u32 variant, u32 shape, const DevJob *jobs, uint32_t cnt, u3
 
 // The shape a launch of this variant actually uses for a requested shape.
 inline u32 br_effective_shape(int logn, u32 variant, u32 shape) {
+    if (variant & BR_V_WIDE) return (u32)br_default_shape(logn);
     if (shape == 0 || logn < 10 || !(variant & BR_V_QLOW1) || shape >= 5 || !br_shape_fits(logn, (int)shape)) return 0;
     return shape;
 }

@@ -693,7 +693,7 @@ template <int LOGN, int TC, bool LAZY>
 struct Product {
     using C = Cfg<LOGN, TC>;
     static constexpr int N = C::N;
-    static constexpr u32 LB = br_qlow1_limb(LAZY);
+    static constexpr u32 LB = br_qlow1_limb(LAZY ? BR_V_LAZY : 0);
     // N = 1024 (lazy keys, Q < 2^54, values below 26.3 Q): the 64-bit sums of
     // limb products hold a whole row, 24 ((26.3 Q >> 28) + 2^28) (2^26 + 2^28) <
     // 2^64, so they stay in registers and are reduced once per row; N = 2048

@@ -70,20 +70,25 @@ __host__ __device__ constexpr u32 ksk_slice_width(u32 n, u32 c0) {
 #define BR_V_LAZY 2u    // correction-free forward NTT with an exact first stage
 #define BR_V_TC1 4u     // leading transform stages on the tensor cores (br_tc.cuh), limb
 #define BR_V_TC2 8u     // configuration 1 or 2
-#define BR_V_ARITH 3u   // the flags of the CUDA-core kernels
+#define BR_V_WIDE 16u   // lazy, Q = c 2^32 + 1, limbs of 30 bits
+#define BR_V_ARITH 19u  // the flags of the CUDA-core kernels
 
 // Limb width of the keys with Q = c 2^32 + 1: 28 bits for the lazy ones (their
 // transform values are below 2^60, their key words below 2^55: a short high
-// key limb lets more products fit 64 bits), 30 for the others.
-__host__ __device__ constexpr u32 br_qlow1_limb(bool lazy) { return lazy ? 28u : 30u; }
+// key limb lets more products fit 64 bits), 30 for the others and for lazy ones
+// whose values pass 15 2^56, where the sum of two 28-bit limbs can exceed 32 bits.
+__host__ __device__ constexpr u32 br_qlow1_limb(u32 variant) {
+    return (variant & (BR_V_LAZY | BR_V_WIDE)) == BR_V_LAZY ? 28u : 30u;
+}
 
 // Arithmetic variant of a key set (BR_V_* flags):
-//  - BR_V_QLOW1: Q = c 2^32 + 1 < 2^60;
+//  - BR_V_QLOW1: Q = c 2^32 + 1 < 2^60, and where the multiply-accumulate takes
+//    the transform's values from, above 2^58 and below 2^60;
 //  - BR_V_LAZY: the correction-free forward transform.  With Q = c 2^32 + 1
-//    it needs (1 + 4 log2 N) Q < 2^62 (its outputs go unreduced into the
-//    multiply-accumulate, whose limbs then stay at most 31 bits) and the
-//    correction-free inverse 128 Q < 2^64; otherwise (1 + 4 log2 N) Q < 2^64
-//    and the exact first stage B + Q B + 4 Q (log2 N - 1) < 2^64 with B < 2^32.
+//    it needs (1 + 4 log2 N) Q <= 2^60 (its outputs go unreduced into the
+//    multiply-accumulate; BR_V_WIDE from 15 2^56 on) and the correction-free
+//    inverse 128 Q < 2^64; otherwise (1 + 4 log2 N) Q < 2^64 and the exact
+//    first stage B + Q B + 4 Q (log2 N - 1) < 2^64 with B < 2^32.
 inline u32 choose_variant(const bm_key_params &p) {
     typedef unsigned __int128 u128;
     u32 logN = 0;
@@ -93,13 +98,13 @@ inline u32 choose_variant(const bm_key_params &p) {
     // (Q < 2^60 keeps every value the Q = c 2^32 + 1 butterflies correct below 2^63)
     bool qlow1 = (p.Q & 0xffffffffull) == 1 && p.Q < (1ull << 60);
     // the Q = c 2^32 + 1 kernels also fix the multiply-accumulate's limbs
-    // (br_qlow1_limb): the transform outputs' bound above 2^58 and below 2^60,
-    // for the lazy ones low enough that their limb sums fit 32 bits
-    const bool lazy1 = (1 + 4 * (u128)logN) * Q < ((u128)15 << 56) && 128 * Q < lim;
-    const u128 xmax1 = lazy1 ? (1 + 4 * (u128)logN) * Q : Q;
+    const u128 xlazy = (1 + 4 * (u128)logN) * Q;
+    const bool lazy1 = xlazy <= ((u128)1 << 60) && 128 * Q < lim;
+    const u128 xmax1 = lazy1 ? xlazy : Q;
     if (qlow1 && !(xmax1 - 1 >= ((u128)1 << 58) && xmax1 - 1 < ((u128)1 << 60))) qlow1 = false;
     if (qlow1) {
         if (lazy1) v |= BR_V_LAZY;
+        if (lazy1 && xlazy >= ((u128)15 << 56)) v |= BR_V_WIDE;
         v |= BR_V_QLOW1;
     } else if ((1 + 4 * (u128)logN) * Q < lim && p.log2_B <= 31 && B + Q * B + 4 * Q * (logN - 1) < lim &&
                128 * Q < lim) {
@@ -111,7 +116,7 @@ inline u32 choose_variant(const bm_key_params &p) {
     // Every such key gains (one bootstrap at N = 1024: 18.7 ms without, 15.9 with
     // them; full blocks as in br_tc.cuh), so no size is left to the other form.
     const bool tc1 = p.Q < (1ull << 54) && p.log2_B <= 9;
-    if ((v & BR_V_QLOW1) && p.l_B <= 6 && p.l_B % 2 == 0 && p.log2_B <= 10 &&
+    if ((v & BR_V_QLOW1) && !(v & BR_V_WIDE) && p.l_B <= 6 && p.l_B % 2 == 0 && p.log2_B <= 10 &&
         ((p.N == 1024 && (v & BR_V_LAZY) && tc1) || p.N == 2048))
         v |= tc1 ? BR_V_TC1 : BR_V_TC2;
     return v;
@@ -135,7 +140,7 @@ inline void limb_plan(const bm_key_params &p, u32 variant, u32 &lbits, u32 &fold
                                             : (u128)p.Q;
     u32 bits = 0;
     while (bits < 66 && ((xmax - 1) >> bits)) bits++;
-    lbits = (variant & BR_V_QLOW1) ? br_qlow1_limb((variant & BR_V_LAZY) != 0) : (bits + 1) / 2;
+    lbits = (variant & BR_V_QLOW1) ? br_qlow1_limb(variant) : (bits + 1) / 2;
     const u128 lim = (u128)1 << lbits;
     const u128 sx = (lim - 1) + ((xmax - 1) >> lbits), sb = (lim - 1) + ((u128)(p.Q - 1) >> lbits);
     const u32 cpb = 512u / (p.N / 16u);     // the largest CPB of any kernel shape
@@ -146,11 +151,11 @@ inline void limb_plan(const bm_key_params &p, u32 variant, u32 &lbits, u32 &fold
 
 // Workspace header: [0] status word, [1 + c] job counter of persistent class c,
 // [BM_WS_GROUP_WORD] job counter of a grouped launch.  Ring degrees 1024, 2048
-// and 4096 have 5, 7 and 4 variants (choose_variant), so a batch has at most 16
+// and 4096 have 6, 8 and 5 variants (choose_variant), so a batch has at most 19
 // persistent classes.
 #define BM_WS_HEADER 256
 #define BM_WS_COUNTER_WORD 1
-#define BM_MAX_CLASSES 16
+#define BM_MAX_CLASSES 19
 #define BM_WS_GROUP_WORD (BM_WS_COUNTER_WORD + BM_MAX_CLASSES)
 static_assert(4 * (BM_WS_GROUP_WORD + 1) <= BM_WS_HEADER, "words of the workspace header");
 

@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(br_shape(SH).threads, 1)
                               const u64 *__restrict__ ct_in, const u32 *__restrict__ luts, u64 *ws,
                               u32 *status, u32 *counter) {
     extern __shared__ __align__(16) u64 sm[];
-    constexpr bool lazy = (V & BR_V_LAZY) != 0, q1 = (V & BR_V_QLOW1) != 0;
+    constexpr bool lazy = (V & BR_V_LAZY) != 0, q1 = (V & BR_V_QLOW1) != 0, wide = (V & BR_V_WIDE) != 0;
     // two slots: thread 0 fetches the next index into one while every thread
     // reads the current one from the other; the barrier that ends each job
     // orders the fetch before the read
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(br_shape(SH).threads, 1)
         const u32 idx = s_next[slot];
         if (idx >= count) break;
         if (threadIdx.x == 0) s_next[slot ^ 1] = atomicAdd(counter, 1u);
-        brk::br_job<LOGN, br_shape(SH).threads, br_shape(SH).rb, lazy, lazy || q1, q1, br_shape(SH).blocks>(
+        brk::br_job<LOGN, br_shape(SH).threads, br_shape(SH).rb, lazy, lazy || q1, q1, br_shape(SH).blocks, wide>(
             jobs[idx], steps, ct_in, luts, ws, status, sm);
         __syncthreads();
         slot ^= 1;
@@ -83,6 +83,9 @@ bm_status launch_variant(u32 variant, u32 shape, const DevJob *d_jobs, uint32_t 
                          const uint64_t *ct_in, const uint32_t *lut, u64 *ws_acc, u32 *status, u32 *counter, int sms,
                          bool dry, cudaStream_t st) {
     switch (variant & BR_V_ARITH) {
+        case BR_V_LAZY | BR_V_QLOW1 | BR_V_WIDE:
+            return launch_class<LOGN, BR_V_LAZY | BR_V_QLOW1 | BR_V_WIDE, br_default_shape(LOGN)>(
+                d_jobs, count, steps, ct_in, lut, ws_acc, status, counter, sms, dry, st);
         case BR_V_LAZY | BR_V_QLOW1:
             return launch_class_shape<LOGN, BR_V_LAZY | BR_V_QLOW1>(shape, d_jobs, count, steps, ct_in, lut, ws_acc,
                                                                    status, counter, sms, dry, st);

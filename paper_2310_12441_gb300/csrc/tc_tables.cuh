@@ -110,7 +110,7 @@ inline std::vector<unsigned char> tc_tables(const bm_key_params &p, u32 variant,
     K.tc_t0 = (u32)(off >> unit) - bias;
     K.tc_m = (u32)(((u128)1 << (unit + 32)) / Q);
     // limb radices of the multiply-accumulate with their Shoup companions
-    const u32 lb = br_qlow1_limb((variant & BR_V_LAZY) != 0);
+    const u32 lb = br_qlow1_limb(variant);
     K.tc_b1 = (1ull << lb) % Q;
     K.tc_b1s = shoup(K.tc_b1);
     K.tc_b2 = (1ull << (2 * lb)) % Q;

@@ -1,5 +1,5 @@
 """A persistent batch with a key of every (ring degree, arithmetic variant)
-class, 16 in one launch sequence: accepted, and the same words as one block per
+class, 19 in one launch sequence: accepted, and the same words as one block per
 job."""
 import numpy as np
 import pytest
@@ -14,11 +14,14 @@ torch = pytest.importorskip("torch")
 Q54, Q60 = P.KEYS_N1024.Q, P.KEYS_N2048.Q          # c 2^32 + 1
 G54, G59 = 18014398509309953, 576460752303415297    # 1 mod 8192, no such form
 
+WIDE = {1024: 28119687757824001, 2048: 25620429108412417, 4096: 23528994783625217}    # lazy, 30-bit limbs
+
 # per ring degree (modulus, digit bits, digits): lazy and corrected transforms
 # with and without the form c 2^32 + 1, then the tensor-core configurations
 COMMON = [(Q54, 15, 4), (Q60, 8, 8), (G54, 9, 6), (G59, 15, 4)]
 CLASSES = [(1024, *k) for k in COMMON + [(Q54, 9, 6)]] + \
-    [(2048, *k) for k in COMMON + [(Q54, 9, 6), (Q54, 10, 6), (Q60, 10, 6)]] + [(4096, *k) for k in COMMON]
+    [(2048, *k) for k in COMMON + [(Q54, 9, 6), (Q54, 10, 6), (Q60, 10, 6)]] + [(4096, *k) for k in COMMON] + \
+    [(N, Q, 10, 6) for N, Q in WIDE.items()]
 
 
 def test_one_key_of_every_class():

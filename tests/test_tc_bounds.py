@@ -11,7 +11,7 @@ import pytest
 from paper_2310_12441_gb300 import build as B
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-LAZY, TC1, TC2 = 2, 4, 8
+Q1, LAZY, TC1, TC2, WIDE = 1, 2, 4, 8, 16
 
 
 def is_prime(n):
@@ -73,3 +73,16 @@ def test_recombination_stays_in_range(prog, N, bits, tc, low, high, end):
         first = (max(e1 + o1, e1 - o0) + 8000) * Q // 1000
         assert first < 2 ** 64
         assert max(2 ** 63, first - 8 * Q) + 8 * Q < 2 ** 64
+
+
+@pytest.mark.parametrize("logN", range(8, 14))
+def test_moduli_of_the_lazy_form_keep_it(prog, logN):
+    """Every modulus c 2^32 + 1 with 2^58 < (1 + 4 log N) Q <= 2^60 has the lazy
+    kernels of that form, with wider limbs from 15 2^56 on."""
+    def variant(Q, bits):
+        return int(subprocess.run([prog, str(1 << logN), str(Q), str(bits)], capture_output=True, text=True,
+                                  check=True).stdout.split()[0])
+    f = 1 + 4 * logN
+    for Q, wide in ((prime_at(2 ** 58 // f + 1, 1), 0), (prime_at(15 * 2 ** 56 // f, -1), 0),
+                    (prime_at(15 * 2 ** 56 // f + 1, 1), WIDE), (prime_at(2 ** 60 // f, -1), WIDE)):
+        assert variant(Q, 15) == Q1 | LAZY | wide
