@@ -25,7 +25,7 @@
 #include "ntt_reg.cuh"
 
 #include "br_launch.cuh"
-#include "ks_tile.cuh"
+#include "ks_plan.cuh"
 
 // ---------------------------------------------------------------------------
 // Sample extraction + key switching
@@ -336,6 +336,7 @@ struct Plan {
     size_t jobs_off, acc_off_bytes, total;
     std::vector<DevJob> dj;
     std::vector<ClassRange> classes;   // persistent classes (order_by_cost plans)
+    std::vector<ksp::Launch> ks;       // the key switch's launches (plan_ks)
     std::vector<u32> gen;     // prefix sums of the jobs' generators, uploaded after the job table
 };
 
@@ -424,7 +425,7 @@ bm_status make_plan(const bm_eval_key *const *keys, const bm_job *jobs, uint32_t
         d.acc_off = acc_words;
         d.variant = choose_variant(k->p);
         limb_plan(k->p, d.variant, d.lbits, d.fold_each);   // lbits as in the key's BSK
-        d.pad = 0;
+        d.key_index = jobs[i].key;
         d.gS = d.gSinv = 0;
         d.gpre = 0;
         if (const uint32_t *u = job_gen(gens, gen_off, i)) {
@@ -590,17 +591,10 @@ struct Fork {
     std::vector<cudaEvent_t> ev;      // [0] fork, [1 + c] join of side stream c
 };
 
-// What the key switch's launch rule needs of a key.
-struct KsKey {
-    const KeyDev *dev;
-    u32 N, n, lks, log2_Bks;
-};
-
 struct KsShape {
     u32 threads, cpt;
     size_t smem;   // digits of all N coefficients (one block per job) + partial sums
     u32 maxN, maxlks, maxn;
-    std::vector<KsKey> keys;
     // shared memory when S blocks split a job's coefficients
     size_t smem_for(u32 S) const { return align_up((size_t)(maxN / S) * maxlks, 16) + 8 * (size_t)(maxn + 1); }
 };
@@ -613,8 +607,6 @@ KsShape ks_shape(const bm_eval_key *const *keys, uint32_t n_keys) {
         maxlks = keys[i]->p.l_ks > maxlks ? keys[i]->p.l_ks : maxlks;
     }
     KsShape k;
-    for (uint32_t i = 0; i < n_keys; i++)
-        k.keys.push_back({keys[i]->d_view, keys[i]->p.N, keys[i]->p.n, keys[i]->p.l_ks, keys[i]->p.log2_Bks});
     k.cpt = maxn + 1 <= 1024 ? 4 : 8;
     k.threads = k.cpt == 4 ? 256 : ((maxn + 1 + 7) / 8 + 31) / 32 * 32;
     k.maxN = maxN;
@@ -622,16 +614,6 @@ KsShape ks_shape(const bm_eval_key *const *keys, uint32_t n_keys) {
     k.maxn = maxn;
     k.smem = k.smem_for(1);
     return k;
-}
-
-// Blocks per job of the key switch: the largest S in {1, 2, 4, 8} with
-// count S <= SMs (one block per job once the batch fills the GPU).
-u32 ks_split(uint32_t count, int device) {
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 1;
-    u32 S = 1;
-    while (S < 8 && (u64)count * (2 * S) <= (u64)sms) S *= 2;
-    return S;
 }
 
 template <auto kern, typename... Args>
@@ -665,44 +647,13 @@ bm_status launch_ks_kernel(uint32_t count, u32 S, const KsShape &ks, cudaStream_
     return BM_OK;
 }
 
-// Samples per thread of the tiled key switch for `count` samples of one key,
-// 0: one block (cluster) per sample.  The cheaper of the two by times measured
-// for l_ks = 3..16, B_ks = 2..128, n = 64..1030, 80..2049 samples, in cycles per
-// coefficient of the ring.  A tile: 700 per stage, 50 and 36 per sample of a
-// thread for every digit, at least its key rows at 64 B per cycle.  A block per
-// sample: per digit 230 (n < 256) or 340, 370 with more blocks than SMs (latency),
-// or for every sample 1/8 per column slice, at least 9/8 (throughput).  Up to
-// half the SMs a cluster per sample is faster (n = 630, N = 1024: 64 samples
-// 0.68 ms against 1.08; 96: 1.32 against 1.08; 2000: 9.6 against 3.2; B_ks = 128,
-// n = 830, N = 256: 300 samples 0.24 against 0.52, 2049: 1.44 against 0.81).
-u32 ks_tile_cpt(const KsKey &k, uint32_t count, u32 sms) {
-    const u32 jn = kst::digits_per_stage(k.lks, k.log2_Bks);
-    if (jn == 0 || 2ull * count <= sms) return 0;
-    const u32 slices = (k.n + kKskCols) / kKskCols, parts = (k.lks + jn - 1) / jn;
-    const u64 fill = (u64)k.lks * ((1u << k.log2_Bks) - 1) * kKskCols * 8 / 64;
-    const u64 latency = count > sms ? 370 : k.n < 256 ? 230 : 340;
-    u64 best_cost = k.lks * std::max<u64>(latency, (u64)count * std::max(slices, 9u) / 8);
-    u32 best = 0;
-    for (u32 cpt = 4; cpt <= kst::kMaxCpt; cpt += 4) {
-        if (kst::smem_bytes(k.lks, k.log2_Bks, cpt * kst::kWarpsPer, 2) > kst::kMaxSmem) break;
-        const u64 tiles = (count + cpt * kst::kWarpsPer - 1) / (cpt * kst::kWarpsPer);
-        const u64 waves = (tiles * slices + sms - 1) / sms;
-        const u64 cost = waves * std::max<u64>(700 * parts + k.lks * (50 + 36 * cpt), fill);
-        if (cost < best_cost) {
-            best_cost = cost;
-            best = cpt;
-        }
-    }
-    return best;
-}
-
 template <auto kern, typename... Args>
-bm_status launch_ks_tile(u32 cpt, const KsKey &k, uint32_t count, cudaStream_t st, Args... args) {
+bm_status launch_ks_tile(u32 cpt, const ksp::Key &k, uint32_t count, cudaStream_t st, Args... args) {
     static std::atomic<uint64_t> attr_done{0};
     bm_status s = ensure_smem(kern, kst::kMaxSmem, attr_done);
     if (s != BM_OK) return s;
-    const u32 slices = (k.n + kKskCols) / kKskCols, per = cpt * kst::kWarpsPer;
-    kern<<<(count + per - 1) / per * slices, kst::kThreads,
+    const u32 per = cpt * kst::kWarpsPer;
+    kern<<<(count + per - 1) / per * ksp::slices(k), kst::kThreads,
            kst::smem_bytes(k.lks, k.log2_Bks, per, kst::stages_of(k.lks, k.log2_Bks, per)), st>>>(args...);
     BM_CUDA_TRY(cudaGetLastError());
     return BM_OK;
@@ -718,48 +669,44 @@ bm_status launch_ks_tile(u32 cpt, const KsKey &k, uint32_t count, cudaStream_t s
         default: return launch_ks_tile<KERN<24>>(24, __VA_ARGS__);             \
     }
 
-bm_status launch_extract_ks_tile(const KsKey &k, u32 cpt, uint32_t count, cudaStream_t st, const DevJob *d_jobs,
-                                 u32 steps, const u64 *ws_acc, uint64_t *d_out, u32 *status) {
-    const u32 slices = (k.n + kKskCols) / kKskCols;
-    BM_KS_TILE(k_extract_keyswitch_tile, cpt, k, count, st, d_jobs, count, slices, steps, ws_acc, d_out, status);
+bm_status launch_extract_ks_tile(const ksp::Launch &l, cudaStream_t st, const DevJob *d_jobs, u32 steps,
+                                 const u64 *ws_acc, uint64_t *d_out, u32 *status) {
+    BM_KS_TILE(k_extract_keyswitch_tile, l.cpt, l.key, l.count, st, d_jobs + l.first, l.count, ksp::slices(l.key), steps,
+               ws_acc, d_out, status);
 }
 
-// Runs of consecutive jobs of one key long enough for the tiles take them, all
-// others the one-block-per-job kernel (neighbouring ones in one launch).
-bm_status launch_extract_ks(const KsShape &ks, const std::vector<DevJob> &dj, int device, cudaStream_t st,
-                            const DevJob *d_jobs, u32 steps, const u64 *ws_acc, uint64_t *d_out, u32 *status) {
-    const uint32_t count = (uint32_t)dj.size();
-    int sms = 0;
-    BM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
-    auto blocks = [&](uint32_t a, uint32_t b) -> bm_status {
-        if (a == b) return BM_OK;
-        const u32 S = ks_split(b - a, device);
-        if (ks.cpt == 4)
-            return launch_ks_kernel<k_extract_keyswitch<4>>(b - a, S, ks, st, d_jobs + a, steps, ws_acc, d_out);
-        return launch_ks_kernel<k_extract_keyswitch<8>>(b - a, S, ks, st, d_jobs + a, steps, ws_acc, d_out);
-    };
-    uint32_t rest = 0;
-    for (uint32_t i = 0, j; i < count; i = j) {
-        for (j = i + 1; j < count && dj[j].key == dj[i].key; j++) {}
-        const KsKey *k = nullptr;
-        for (const KsKey &x : ks.keys)
-            if (x.dev == dj[i].key) k = &x;
-        const u32 cpt = k ? ks_tile_cpt(*k, j - i, (u32)sms) : 0;
-        if (!cpt) continue;
-        bm_status s = blocks(rest, i);
-        if (s != BM_OK) return s;
-        if ((s = launch_extract_ks_tile(*k, cpt, j - i, st, d_jobs + i, steps, ws_acc, d_out, status)) !=
-            BM_OK) return s;
-        rest = j;
+// The key switch's launches for the plan's jobs (in plan order).
+void plan_ks(Plan &pl, const bm_eval_key *const *keys, u32 sms) {
+    std::vector<ksp::Run> runs;
+    const DevJob *prev = nullptr;
+    for (const DevJob &d : pl.dj) {
+        const bm_key_params &p = keys[d.key_index]->p;
+        if (prev && prev->key == d.key) runs.back().count++;
+        else runs.push_back({1, {p.N, p.n, p.l_ks, p.log2_Bks}});
+        prev = &d;
     }
-    return blocks(rest, count);
+    pl.ks = ksp::plan(runs, sms);
+}
+
+bm_status launch_extract_ks(const KsShape &ks, const std::vector<ksp::Launch> &plan, u32 sms, cudaStream_t st,
+                            const DevJob *d_jobs, u32 steps, const u64 *ws_acc, uint64_t *d_out, u32 *status) {
+    for (const ksp::Launch &l : plan) {
+        const u32 S = ksp::split(l.count, sms);
+        bm_status s = BM_OK;
+        if (l.cpt) s = launch_extract_ks_tile(l, st, d_jobs, steps, ws_acc, d_out, status);
+        else if (ks.cpt == 4)
+            s = launch_ks_kernel<k_extract_keyswitch<4>>(l.count, S, ks, st, d_jobs + l.first, steps, ws_acc, d_out);
+        else s = launch_ks_kernel<k_extract_keyswitch<8>>(l.count, S, ks, st, d_jobs + l.first, steps, ws_acc, d_out);
+        if (s != BM_OK) return s;
+    }
+    return BM_OK;
 }
 
 // Every launch of one batch (the plan is already in the workspace).
 // Largest thread-block cluster (blocks per job) a grouped launch may use.
 constexpr u32 kMaxCluster = 8;
 
-bm_status launch_all(const Plan &pl, uint32_t n_persistent, const KsShape &ks, int device, u32 steps, bool do_ks,
+bm_status launch_all(const Plan &pl, uint32_t n_persistent, const KsShape &ks, int device, u32 sms, u32 steps, bool do_ks,
                      const uint64_t *d_ct_in, const uint32_t *d_lut, uint64_t *d_out, char *ws,
                      cudaStream_t st, const Shapes &shapes, u32 max_cluster = kMaxCluster,
                      const Fork *fork = nullptr) {
@@ -788,7 +735,7 @@ bm_status launch_all(const Plan &pl, uint32_t n_persistent, const KsShape &ks, i
     if ((s = run_groups(pl, n_persistent, count, steps, d_ct_in, d_lut, ws, st, false, max_cluster, shapes)) != BM_OK)
         return s;
     if (do_ks) {
-        if ((s = launch_extract_ks(ks, pl.dj, device, st, d_jobs, steps, ws_acc, d_out, (u32 *)ws)) != BM_OK)
+        if ((s = launch_extract_ks(ks, pl.ks, sms, st, d_jobs, steps, ws_acc, d_out, (u32 *)ws)) != BM_OK)
             return s;
     } else {
         k_copy_acc<<<count, 256, 0, st>>>(d_jobs, steps, ws_acc, d_out);
@@ -850,7 +797,10 @@ static bm_status bootstrap_impl(const bm_eval_key *const *keys, uint32_t n_keys,
     cudaStream_t st = (cudaStream_t)stream;
     char *ws = (char *)d_ws;
     if ((s = upload_plan(pl, ws, st)) != BM_OK) return s;
-    return launch_all(pl, 0, ks_shape(keys, n_keys), dev, steps, do_ks, d_ct_in, d_lut, d_out, ws, st,
+    int sms = 0;
+    BM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (do_ks) plan_ks(pl, keys, (u32)sms);
+    return launch_all(pl, 0, ks_shape(keys, n_keys), dev, (u32)sms, steps, do_ks, d_ct_in, d_lut, d_out, ws, st,
                       Shapes::current());
 }
 
@@ -955,12 +905,11 @@ extern "C" bm_status bm_key_switch(const bm_eval_key *key, const uint64_t *d_lwe
     cudaStream_t st = (cudaStream_t)stream;
     int sms = 0;
     BM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, key->device));
-    const KsKey &k = ks.keys[0];
-    if (const u32 cpt = ks_tile_cpt(k, count, (u32)sms)) {
-        const u32 slices = (k.n + kKskCols) / kKskCols;
-        BM_KS_TILE(k_key_switch_tile, cpt, k, count, st, key->d_view, count, slices, d_lwe_in, d_out);
+    const ksp::Key k{key->p.N, key->p.n, key->p.l_ks, key->p.log2_Bks};
+    if (const u32 cpt = ksp::tile_cpt(k, count, (u32)sms)) {
+        BM_KS_TILE(k_key_switch_tile, cpt, k, count, st, key->d_view, count, ksp::slices(k), d_lwe_in, d_out);
     }
-    const u32 S = ks_split(count, key->device);
+    const u32 S = ksp::split(count, (u32)sms);
     if (ks.cpt == 4) return launch_ks_kernel<k_key_switch<4>>(count, S, ks, st, key->d_view, d_lwe_in, d_out);
     return launch_ks_kernel<k_key_switch<8>>(count, S, ks, st, key->d_view, d_lwe_in, d_out);
 }
@@ -1120,7 +1069,7 @@ extern "C" bm_status bm_modmul_peak(int device, uint32_t iters, double *rate) {
 extern "C" void bm_batch_free(bm_batch *b);
 
 struct bm_batch {
-    int device;
+    int device, sms;
     uint32_t flags, n_persistent;
     Plan pl;
     Fork fork;
@@ -1154,6 +1103,11 @@ extern "C" bm_status bm_batch_create(const bm_eval_key *const *keys, uint32_t n_
     }
     b->n_persistent = (flags & BM_BATCH_PERSISTENT) ? persistent_prefix(b->pl) : 0;
     b->ks = ks_shape(keys, n_keys);
+    if (cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        delete b;
+        return BM_ECUDA;
+    }
+    plan_ks(b->pl, keys, (u32)b->sms);
     b->shapes = Shapes::current();
     b->d_ct_in = d_ct_in;
     b->d_lut = d_lut;
@@ -1197,13 +1151,13 @@ extern "C" bm_status bm_batch_run(bm_batch *b, void *stream) {
     DeviceGuard g(b->device);
     cudaStream_t st = (cudaStream_t)stream;
     if (!(b->flags & BM_BATCH_GRAPH))
-        return launch_all(b->pl, b->n_persistent, b->ks, b->device, 0xffffffffu, true, b->d_ct_in, b->d_lut,
+        return launch_all(b->pl, b->n_persistent, b->ks, b->device, (u32)b->sms, 0xffffffffu, true, b->d_ct_in, b->d_lut,
                           b->d_out, b->ws, st, b->shapes, b->max_cluster(), &b->fork);
     if (!st) return BM_EINVAL;   // the legacy default stream cannot be captured
     if (!b->exec) {
         cudaGraph_t graph = nullptr;
         BM_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        bm_status s = launch_all(b->pl, b->n_persistent, b->ks, b->device, 0xffffffffu, true, b->d_ct_in,
+        bm_status s = launch_all(b->pl, b->n_persistent, b->ks, b->device, (u32)b->sms, 0xffffffffu, true, b->d_ct_in,
                                  b->d_lut, b->d_out, b->ws, st, b->shapes, b->max_cluster(), &b->fork);
         cudaError_t e = cudaStreamEndCapture(st, &graph);
         if (s != BM_OK) {

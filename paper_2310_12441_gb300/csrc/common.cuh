@@ -48,7 +48,7 @@ struct DevJob {
     u32 fold_each;     // 1: a batch's limb products may exceed 64 bits, fold per combo
     u32 gS;            // generator: 0 for P(1) of Example 1, else S = sum u mod 2N (odd)
     u32 gSinv;         // S^-1 mod 2N
-    u32 pad;
+    u32 key_index;     // of the call's keys (host only)
     u64 gpre;          // u32 offset from the workspace start of the prefix sums
                        // pre[k] = (u_0 + ... + u_{k-1}) mod 2N, k in [0, m] (gS != 0)
 };
