@@ -39,25 +39,29 @@ inline u32 split(u64 count, u32 sms) {
 // samples of one key.  Per coefficient of the ring, a tile: 700 per stage, 50 and
 // 36 per sample of a thread for every digit, at least its key rows at 64 B per
 // cycle.  A block per sample: per digit 230 (n < 256) or 340, 370 with more
-// blocks than SMs (latency, shared by the blocks of a cluster), or for every
+// blocks than SMs, 900 with more than the three an SM holds (latency, shared by
+// the blocks of a cluster), or for every
 // sample 1/8 per column slice, at least 9/8 (throughput).  (n = 630, N = 1024: 64
 // samples 0.68 ms against 1.08 in tiles; 96: 1.32 against 1.08; 2000: 9.6 against
 // 3.2; B_ks = 128, n = 830, N = 256: 300 samples 0.24 against 0.52, 2049: 1.44
 // against 0.81.)
 struct Blocks {        // one launch of a block or cluster per sample
-    u64 count = 0, thr = 0, few = 0, many = 0;      // few, many: latency up to and above SMs samples
+    u64 count = 0, thr = 0, few = 0, many = 0, waves = 0;      // latency up to SMs, 3 SMs samples, above
     void add(const Key &k, u64 samples) {
         const u64 digits = (u64)k.N * k.lks;
         add(Blocks{samples, k.N * (k.lks * (samples * std::max(slices(k), 9u) / 8)), digits * (k.n < 256 ? 230 : 340),
-             digits * 370});
+             digits * 370, digits * 900});
     }
     void add(const Blocks &b) {
         count += b.count;
         thr += b.thr;
         few = std::max(few, b.few);
         many = std::max(many, b.many);
+        waves = std::max(waves, b.waves);
     }
-    u64 cost(u32 sms) const { return std::max(thr, (count > sms ? many : few) / split(count, sms)); }
+    u64 cost(u32 sms) const {
+        return std::max(thr, (count > 3ull * sms ? waves : count > sms ? many : few) / split(count, sms));
+    }
 };
 
 constexpr u64 kLaunch = 5000;     // a launch more on the stream
