@@ -336,9 +336,13 @@ bm_status bm_bootstrap_arbitrary(const bm_eval_key *key, uint32_t m, uint32_t t,
  *   3: radix 8, 512 threads, 2 blocks/SM     (N = 1024)
  *   4: radix 8, 512 threads, 1 block/SM      (N = 1024..4096)
  * Shapes 1..4 are compiled for keys whose Q = c 2^32 + 1; other keys run
- * shape 0.  At N = 1024 (Q < 2^54) and 2048 shape 1 runs such keys with even
- * l_B <= 6 and log2_B <= 10 (9 at N = 1024) with the leading transform stages
- * on the tensor cores (640 threads, 1 block/SM).  bm_kernel_shape_info describes shape s at ring degree N
+ * shape 0, and those with (1 + 4 log2 N) Q within 6% below 2^60 the default
+ * shape.  Keys of that form with l_B = 6 and 9-bit digits (N = 1024 and 2048,
+ * Q < 2^54) or 10-bit ones (N = 2048) run shape 1 with the leading transform
+ * stages on the tensor cores: 640 threads, 1 block/SM, a block alternating
+ * between two jobs, under BM_BATCH_ONE_BLOCK too.  (At N = 2048 with Q < 2^54.4,
+ * launches that give a block one job of fewer than eight rows do not.)
+ * bm_kernel_shape_info describes shape s without them at ring degree N
  * (BM_EINVAL when it does not fit).  bm_set_kernel_shape selects the shape
  * that later launches at ring degree N use (BM_SHAPE_DEFAULT: the built-in
  * choice, shape 1 for N = 1024..8192 and 0 below); reusable batches keep the shapes current at bm_batch_create.

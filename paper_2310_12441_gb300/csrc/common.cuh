@@ -110,13 +110,13 @@ inline u32 choose_variant(const bm_key_params &p) {
                128 * Q < lim) {
         v |= BR_V_LAZY;
     }
-    // The tensor-core stages (br_tc.cuh): digits of at most 10 bits (9 at N =
-    // 1024), the digits of two (sign, component) pairs (N = 1024) or one (N =
-    // 2048) in whole half batches, within the shared memory beside the weights.
-    // Every such key gains (one bootstrap at N = 1024: 18.7 ms without, 15.9 with
-    // them; full blocks as in br_tc.cuh), so no size is left to the other form.
+    // The tensor-core stages (br_tc.cuh): digits of 9 bits (configuration 1) or, at
+    // N = 2048, 10 (2), six of them: with Q above 2^52.5 (the form's lower bound)
+    // and 2^(6 log2 B) >= Q, other l_B or fewer bits do not occur.  Every such key
+    // gains (one bootstrap at N = 1024: 18.7 ms without, 15.9 with them; full blocks
+    // as in br_tc.cuh) but for small launches of lazy ones at N = 2048 (launch_tc).
     const bool tc1 = p.Q < (1ull << 54) && p.log2_B <= 9;
-    if ((v & BR_V_QLOW1) && !(v & BR_V_WIDE) && p.l_B <= 6 && p.l_B % 2 == 0 && p.log2_B <= 10 &&
+    if ((v & BR_V_QLOW1) && !(v & BR_V_WIDE) && p.l_B == 6 && p.log2_B <= 10 &&
         ((p.N == 1024 && (v & BR_V_LAZY) && tc1) || p.N == 2048))
         v |= tc1 ? BR_V_TC1 : BR_V_TC2;
     return v;
@@ -229,7 +229,8 @@ bm_status bm_launch_br_big(u32 N, const DevJob *jobs, uint32_t cnt, u32 steps, c
 
 // Tensor-core form (br_tc.cu), ring degrees 1024 and 2048 of keys with a
 // BR_V_TC* flag: grouped launches and persistent classes (max_cluster = 1);
-// counter: the jobs' counter, a word of the workspace header; sms 0: look up.
+// counter: the jobs' counter, a word of the workspace header; sms: 0 for grouped
+// launches (looked up), which may take the CUDA-core kernel after all (launch_tc).
 bm_status bm_launch_br_tc(u32 N, u32 variant, const DevJob *jobs, uint32_t cnt, u32 mmax, u32 max_cluster, u32 steps,
                           const uint64_t *ct_in, const uint32_t *lut, u64 *ws_acc, u32 *status, u32 *counter, int sms,
                           cudaStream_t st, bool dry);
