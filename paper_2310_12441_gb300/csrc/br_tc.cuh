@@ -1093,8 +1093,10 @@ __device__ __forceinline__ void product_warps(Shared &sh, unsigned char *sm, con
                     }
                     if (bar_or(sh)) break;
                     if (!sl[cs].on) {
-                        fill(cs);
+                        // (a job that has waited for its key comes before new
+                        // ones: they are in order of cost)
                         fill(cs ^ 1);
+                        fill(cs);
                     }
                     if (!ahead) {
                         if (!sl[ns].on) ns = cs ^ 1;

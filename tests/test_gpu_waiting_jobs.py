@@ -1,0 +1,51 @@
+"""A job that waits in its block for another key's job to end starts next, not
+after all others: one long job of a second key among jobs of a first takes as
+long as when all have one key."""
+import numpy as np
+import pytest
+
+from paper_2310_12441_gb300 import params as P
+from paper_2310_12441_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def test_long_job_of_a_second_key():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2310_12441_gb300 import api
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    K = P.KEYS_N1024
+    kp = P.KeyParams(n=30, N=K.N, Q=K.Q, log2_B=K.log2_B, l_B=K.l_B, log2_Bks=4, l_ks=2)
+    eks = [api.bm_keygen_seeded(kp, 70 + i)[1] for i in range(2)]
+    # a long job for every block, one more of them, then eight short ones per block:
+    # 16 rows per block, 24 where the one more comes last
+    m = np.r_[np.full(sms + 1, 8), np.full(8 * sms, 1)]
+    count, t, W = len(m), 64, kp.n + 1
+    rng = np.random.default_rng(2)
+    ct = np.stack([rng.integers(0, 2 * kp.N * int(x), W, dtype=np.uint64) for x in m])
+    luts, _ = synth.luts(t, count, 3, mix="mixed")
+    d_in, d_lut = api.to_device_u64(ct.ravel()), api.to_device_u32(luts.ravel())
+    best = []
+    for second in (0, 1):
+        ki = np.zeros(count, int)
+        ki[sms] = second
+        jobs = api.make_jobs(ki, 1, t, np.arange(count) * W, np.arange(count) * t, np.arange(count) * W)
+        jobs["m"] = m
+        out = torch.zeros(count * W, dtype=torch.int64, device="cuda")
+        ws = api.workspace(api.bm_workspace_bytes(eks, jobs))
+        b = api.Batch(eks, jobs, d_in, d_lut, out, ws, api.BATCH_PERSISTENT)
+        ms = []
+        for _ in range(6):
+            t0, t1 = torch.cuda.Event(True), torch.cuda.Event(True)
+            t0.record()
+            b.run()
+            t1.record()
+            torch.cuda.synchronize()
+            ms.append(t0.elapsed_time(t1))
+        assert api.bm_workspace_status(ws) == 0
+        b.free()
+        best.append(min(ms))
+    assert best[1] < 1.25 * best[0]
