@@ -217,11 +217,12 @@ __device__ __forceinline__ void ksk_row(size_t row, GetA get_a, int ev, const in
     const u32 lane = threadIdx.x & 31;
     const u32 n = K.n, B1 = (1u << K.log2_Bks) - 1;
     const u64 Q = K.mq.Q;
-    const u32 rows = K.l_ks * B1, r = (u32)(row % rows);
-    u64 *o = ksk + row / rows * rows * ksk_pitch(n);
+    // (rows in all below 2^32: at most 1275 per coefficient)
+    const u32 rows = K.l_ks * B1, i = (u32)row / rows, r = (u32)row - i * rows;
+    u64 *o = ksk + (size_t)i * rows * ksk_pitch(n);
     auto at = [&](u32 c) -> u64 & {
         const u32 c0 = c & ~(kKskCols - 1);
-        return o[(size_t)c0 * rows + (size_t)r * ksk_slice_width(n, c0) + c - c0];
+        return o[c0 * rows + r * ksk_slice_width(n, c0) + c - c0];
     };
     u64 lo = 0, hi = 0;
     for (u32 c = lane; c < n; c += 32) {
@@ -234,9 +235,7 @@ __device__ __forceinline__ void ksk_row(size_t row, GetA get_a, int ev, const in
     u64 acc = reduce128(lo, hi, K.mq);
     for (int off = 16; off; off >>= 1) acc = add_mod(acc, __shfl_down_sync(0xffffffffu, acc, off), Q);
     if (lane == 0) {
-        const u32 v = (u32)(row % B1) + 1;
-        const u32 j = (u32)((row / B1) % K.l_ks);
-        const u32 i = (u32)(row / ((size_t)B1 * K.l_ks));
+        const u32 j = r / B1, v = r - j * B1 + 1;
         u64 l2 = 0, h2 = 0;
         mac128(l2, h2, v, G.g[j]);
         u64 vg = reduce128(l2, h2, K.mq);

@@ -120,8 +120,15 @@ inline std::vector<unsigned char> tc_tables(const bm_key_params &p, u32 variant,
     K.tc_fsh = 0;
     while ((2ull << K.tc_fsh) < c1) K.tc_fsh++;
     K.tc_fs = (u32)(((u128)1 << (32 + K.tc_fsh)) / c1);
+    // (8192 powers and 40960 or more limbs: Shoup products and looked-up halves
+    // instead of 128-bit divisions and conversions)
+    uint16_t half[2049];       // -1024 .. 1024 in fp16
+    for (int v = -1024; v <= 1024; v++) {
+        const __half h = __float2half((float)v);
+        memcpy(&half[v + 1024], &h, 2);
+    }
     for (u32 c = 0; c < 64; c++) {
-        const u64 w = tab[64 + c], w2 = mulmod(w, w);
+        const u64 w = tab[64 + c], w2 = mulmod(w, w), w2s = shoup(w2);
         u64 f[2] = {1 % Q, w};
         u128 sum[2] = {0, 0};
         for (u32 i = 0; i < 64; i++) {
@@ -134,10 +141,11 @@ inline std::vector<unsigned char> tc_tables(const bm_key_params &p, u32 variant,
                         r = ((v + (1 << (R - 1))) & ((1 << R) - 1)) - (1 << (R - 1));
                         v = (v - r) >> R;
                     }
-                    const __half h = __float2half((float)r);
-                    memcpy(&out[(e * NL + l) * 8192 + (c / 8) * 1024 + (i / 8) * 128 + (c % 8) * 16 + (i % 8) * 2], &h, 2);
+                    memcpy(&out[(e * NL + l) * 8192 + (c / 8) * 1024 + (i / 8) * 128 + (c % 8) * 16 + (i % 8) * 2],
+                           &half[r + 1024], 2);
                 }
-                f[e] = mulmod(f[e], w2);
+                const u64 x = f[e] * w2 - (u64)(((u128)f[e] * w2s) >> 64) * Q;
+                f[e] = x >= Q ? x - Q : x;
             }
         }
         for (u32 e = 0; e < 2; e++) {
