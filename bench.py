@@ -63,13 +63,22 @@ def kernel_hash():
     return h.hexdigest()[:16]
 
 
-def modmuls_per_bootstrap(kp, m):
-    """Algorithmic 64-bit modular multiplications of one bootstrap: per CMux
-    step and row, 4 l_B forward and 2 inverse negacyclic NTTs of (N/2) log2 N
-    butterflies, and 8 l_B N multiply-accumulates against the key."""
+def tensor_form(kp):
+    """Whether full launches at kernel shape 1 run these keys' leading seven
+    forward stages on the tensor cores (k_blind_rotate_tc): six digits of 9
+    bits, at N = 2048 also 10, and Q = c 2^32 + 1."""
+    return kp.Q % 2 ** 32 == 1 and kp.l_B == 6 and (kp.N, kp.log2_B) in ((1024, 9), (2048, 9), (2048, 10))
+
+
+def modmuls_per_bootstrap(kp, m, tensor=False):
+    """64-bit modular multiplications of one bootstrap: per CMux step and row,
+    4 l_B forward and 2 inverse negacyclic NTTs of (N/2) log2 N butterflies, and
+    8 l_B N multiply-accumulates against the key.  tensor: without the seven
+    forward stages that the tensor cores do."""
     import math
     N, lB = kp.N, kp.l_B
-    return kp.n * m * ((4 * lB + 2) * (N // 2) * int(math.log2(N)) + 8 * lB * N)
+    fwd = int(math.log2(N)) - (7 if tensor else 0)
+    return kp.n * m * ((4 * lB * fwd + 2 * int(math.log2(N))) * (N // 2) + 8 * lB * N)
 
 
 class ClockSampler:
@@ -249,8 +258,8 @@ def count_failures(api, sk, w, batches):
 
 def kernel_roofline(api, ek, w, jobs, batch, ws, stream, flush, dev, peak, reps=3):
     """Blind rotation alone (bm_blind_rotate, same jobs and launch shape)
-    timed with CUDA events on its stream: algorithmic modmuls / time against
-    the measured modmul peak."""
+    timed with CUDA events on its stream: modmuls of the CUDA cores / time
+    against the measured modmul peak."""
     import torch
     kp, m = w.keys, w.shape.m
     count = len(jobs)
@@ -267,16 +276,19 @@ def kernel_roofline(api, ek, w, jobs, batch, ws, stream, flush, dev, peak, reps=
         torch.cuda.synchronize(dev)
         ts.append(a.elapsed_time(b))
     del d_acc
-    mm = modmuls_per_bootstrap(kp, m) * count
+    shape = api.get_kernel_shape(kp.N)
+    tensor = shape == 1 and tensor_form(kp)
+    mm = modmuls_per_bootstrap(kp, m, tensor) * count
     rot_s = float(np.mean(ts)) * 1e-3
     traffic = None
     cap = CAPTURED_TRAFFIC.get(w.name)
     if cap and kernel_hash() == cap["hash"]:
         traffic = cap["bytes_per_job"] * count
-    shape = api.get_kernel_shape(kp.N)
-    radix, threads, blocks = api.kernel_shapes(kp.N)[shape]
+    radix, threads, blocks = (8, 640, 1) if tensor else api.kernel_shapes(kp.N)[shape]
     return {"bound": "alu", "achieved": mm / rot_s / 1e9, "peak": peak / 1e9, "unit": "Gmodmul/s",
-            "frac": (mm / rot_s) / peak, "traffic": traffic, "kernel": "k_blind_rotate",
+            "frac": (mm / rot_s) / peak, "traffic": traffic,
+            "kernel": "k_blind_rotate_tc" if tensor else "k_blind_rotate",
+            "not_counted": "seven of the forward stages (tensor cores), recombination of their limbs" if tensor else "",
             "shape": {"id": shape, "ntt_radix": radix, "threads": threads, "blocks_per_sm": blocks},
             "kernel_ms": rot_s * 1e3, "modmuls_per_launch": mm,
             "peak_kind": "measured: the blind rotation's own modular product in a throughput loop"}
@@ -549,7 +561,8 @@ def run_extras(args, api, dev, stream, flush, peak):
     ws = api.workspace(api.bm_workspace_bytes(keys, bu.jobs), dev)
     tuned = autotune.tune(ksets, bu.jobs, d_in, d_lut, d_out, ws, stream, use_cache=False)
     modes = {}
-    mm = sum(modmuls_per_bootstrap(ksets[int(j["key"])].kp, int(j["m"])) for j in bu.jobs)
+    mm = sum(modmuls_per_bootstrap(ksets[int(j["key"])].kp, int(j["m"]), tensor_form(ksets[int(j["key"])].kp))
+             for j in bu.jobs)
     for name, fl in autotune.CANDIDATES.items():
         b = api.Batch(keys, bu.jobs, d_in, d_lut, d_out, ws, fl)
         b.run(stream)

@@ -6,7 +6,8 @@ oracle):
 
   * the kernel shape of each ring degree in the batch (bm_kernel_shape_info:
     NTT radix 16 or 8, 256 / 512 / 1024 threads per block, one or two blocks
-    per SM), timed on a sample of the batch's jobs of that degree;
+    per SM), timed on a sample of the batch's jobs of that degree (shape 1 of
+    keys with tensor-core stages runs 640 threads; "desc" gives the CUDA-core form);
   * the launch mode: "grouped" (one launch per run of equal degree and
     arithmetic variant, one after the other) or "persistent" (one persistent
     kernel per such class, the classes running concurrently), timed on the

@@ -298,7 +298,7 @@ __global__ void k_lwe_sub(const u64 *__restrict__ x, const u64 *__restrict__ y, 
 
 // Throughput probe of the blind rotation's own modular product: the
 // three-product Shoup multiplication for Q = c 2^32 + 1 (shoup3_qlow1_lazy:
-// seven multiplier instructions, 22 multiplier-pipe cycles per warp), eight
+// seven multiplier instructions, 23 multiplier-pipe cycles per warp), eight
 // independent chains per thread; every output in [0, 4Q) is a valid next
 // input.
 __global__ void k_modmul_probe(u64 *out, u32 iters, u32 c, u64 w, u64 wsh) {

@@ -356,9 +356,10 @@ __device__ __forceinline__ void digit_warps(Shared &sh, unsigned char *sm, u32 c
         if constexpr (LOGN == 10) {
             // A few clusters walk the key, larger than the L2, one step's rows at
             // a time and at HBM latency: the launch's blocks bring the next
-            // step's rows to the L2, 1 KB each in turn (one job of 630 steps 17.1
-            // -> 15.7 ms, 30 jobs 16.4 -> 15.7; at N = 2048 the loads are
-            // spread over twice the work and it costs 1%).
+            // step's rows to the L2, 1 KB each in turn (30 jobs of 630 steps 16.4
+            // -> 15.7 ms; one job 15.7, without it 15.4 to 17.1 by where the key
+            // lies; at N = 2048 the loads are spread over twice the work and it
+            // costs 1%).
             if (csize > 1 && un.row == 0 && un.part == 0 && s.k + 1 < s.steps) {
                 const u32 chunks = 4 * lB * 2 * N * 8 / 1024;
                 const unsigned char *next = (const unsigned char *)(K->bsk + (size_t)(s.k + 1) * 4 * lB * 2 * N);
