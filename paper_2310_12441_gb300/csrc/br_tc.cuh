@@ -37,14 +37,16 @@
 // inverse transforms and digits at a job's step boundary overlap the other
 // job's transforms; blocks take further jobs from a counter.
 //
-// What bounds it: the 32-bit multiplier pipe (recombination, three or four
-// remaining stages, multiply-accumulate, inverse transforms), 68% busy with two
-// jobs in every block (61% with one) against 59% (50%) of the issue slots and
-// 10% of the tensor pipe; at N = 2048 the transform warps' integer instructions.
+// What bounds it: at N = 1024 the 32-bit multiplier pipe (recombination, three
+// remaining stages, multiply-accumulate, inverse transforms), 67% busy with two
+// jobs in every block (63% with one) against 54% (51%) of the issue slots and 11%
+// of the tensor pipe.  At N = 2048 no unit: multiplier and issue slots read 52%
+// with one job or two, and long scoreboard (key rows and accumulators from the
+// L2, TMEM) leads the stalls, so the roles wait for one another.
 // Per row of one CMux step and SM, blocks full: N = 1024, Q < 2^54: 24.9 us with
 // all stages in the CUDA cores (br_job), 16.7 us here; N = 2048, Q < 2^60: 64.2
-// and 56.3 us.  1000 bootstraps at N = 1024 with m = 4: 444 and 313 ms; 200 at
-// N = 2048 with m = 8: 579 and 511 ms.
+// and 56.3 us.  1000 bootstraps at N = 1024 with m = 4: 444 and 312 ms; 200 at
+// N = 2048 with m = 8: 579 and 512 ms.
 #pragma once
 #include "blind_rotate.cuh"
 #include "tc_tables.cuh"

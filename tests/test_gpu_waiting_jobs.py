@@ -49,3 +49,41 @@ def test_long_job_of_a_second_key():
         b.free()
         best.append(min(ms))
     assert best[1] < 1.25 * best[0]
+
+
+def test_order_of_uneven_jobs():
+    """A grouped batch takes as long in any order of its jobs as longest first."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2310_12441_gb300 import api
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    K = P.KEYS_N2048
+    kp = P.KeyParams(n=20, N=K.N, Q=K.Q, log2_B=K.log2_B, l_B=K.l_B, log2_Bks=4, l_ks=2)
+    ek = api.bm_keygen_seeded(kp, 75)[1]
+    m = np.random.default_rng(1).choice([2, 4, 8], 4 * sms)
+    count, t, W = len(m), 64, kp.n + 1
+    rng = np.random.default_rng(4)
+    ct = np.stack([rng.integers(0, 2 * kp.N * int(x), W, dtype=np.uint64) for x in m])
+    luts, _ = synth.luts(t, count, 3, mix="mixed")
+    d_in, d_lut = api.to_device_u64(ct.ravel()), api.to_device_u32(luts.ravel())
+    jobs = api.make_jobs(0, 1, t, np.arange(count) * W, np.arange(count) * t, np.arange(count) * W)
+    jobs["m"] = m
+    best, outs = [], []
+    for order in (np.argsort(-m, kind="stable"), np.arange(count)):
+        out = torch.zeros(count * W, dtype=torch.int64, device="cuda")
+        ws = api.workspace(api.bm_workspace_bytes([ek], jobs[order]))
+        b = api.Batch([ek], jobs[order], d_in, d_lut, out, ws, 0)
+        ms = []
+        for _ in range(6):
+            t0, t1 = torch.cuda.Event(True), torch.cuda.Event(True)
+            t0.record()
+            b.run()
+            t1.record()
+            torch.cuda.synchronize()
+            ms.append(t0.elapsed_time(t1))
+        assert api.bm_workspace_status(ws) == 0
+        b.free()
+        best.append(min(ms))
+        outs.append(out)
+    assert torch.equal(outs[0], outs[1])
+    assert best[1] < 1.15 * best[0]
