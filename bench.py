@@ -45,12 +45,12 @@ METRIC = "bootstraps/s on 1 GB300 (batched vs plain, bit-exact); p50/p99 served 
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the
 # blind-rotation kernel per job, from one ncu capture of a 152-job launch of
-# the workload (command: bench.py --workload <name> --count 152 under
-# `ncu --set full -k regex:k_blind_rotate`), valid while the kernel sources
-# hash to the captured version.
+# the workload, all its steps (`ncu --metrics dram__bytes_read.sum,
+# dram__bytes_write.sum -k regex:k_blind_rotate`), valid while the kernel
+# sources hash to the captured version.
 KERNEL_SOURCES = ["blind_rotate.cuh", "br_tc.cuh", "tc_tables.cuh", "br_tc.cu", "ntt_reg.cuh", "modarith.cuh", "common.cuh", "br_launch.cuh"]
 CAPTURED_TRAFFIC = {
-    P.BATCH_N1024.name: {"hash": "2e5795488aa486bf", "bytes_per_job": (254.637056e6 + 6.749184e6) / 152},
+    P.BATCH_N1024.name: {"hash": "61fb3dd6c36c8c57", "bytes_per_job": (253.93e6 + 4.12e6) / 152},
 }
 
 
