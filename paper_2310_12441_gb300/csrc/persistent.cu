@@ -110,9 +110,14 @@ bm_status bm_launch_persistent_class(u32 N, u32 variant, u32 shape, const DevJob
                                      u32 *status, u32 *counter, int device, bool dry, cudaStream_t st) {
     int sms = 0;
     BM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
-    if (shape == 1 && (variant & (BR_V_TC1 | BR_V_TC2)))
-        return bm_launch_br_tc(N, variant, d_jobs, count, 1, 1, steps, ct_in, lut, ws_acc, status, counter, sms, st,
-                               dry);
+    // lazy keys of configuration 2 without a second job for any block stay on the
+    // CUDA cores (24 steps, 152 jobs: m = 1 1.86 ms, 1.89 there; m = 2 3.12 and 3.17)
+    const bool alone = (variant & BR_V_TC2) && (variant & BR_V_LAZY) && !dry && count <= (uint32_t)sms;
+    if (shape == 1 && (variant & (BR_V_TC1 | BR_V_TC2)) && !alone) {
+        const bm_status s = bm_launch_br_tc(N, variant, d_jobs, count, 1, 1, steps, ct_in, lut, ws_acc, status, counter,
+                                            sms, st, dry);
+        if (s != BM_OK || !dry) return s;      // (dry: the attributes of either kernel)
+    }
     switch (N) {
         case 1024:
             return launch_variant<10>(variant, shape, d_jobs, count, steps, ct_in, lut, ws_acc, status, counter, sms,
